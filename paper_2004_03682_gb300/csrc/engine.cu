@@ -525,13 +525,7 @@ void permute_into(Ctx& c, const std::string& site, Tensor& dst, const char* dl, 
 // over the symmetry blocks (all instances).
 GemmPlan make_gemm_plan(Ctx& c, const Layout& A, const Layout& B, const Layout& C) {
   GemmPlan g;
-  int64_t tiles_mn = 0;
-  int64_t maxM = 0, maxN = 0;
-  for (int q = 0; q < c.G; ++q) {
-    if (A.rows[q] && B.cols[q]) { maxM = std::max<int64_t>(maxM, A.rows[q]); maxN = std::max<int64_t>(maxN, B.cols[q]); }
-  }
-  g.tm = maxM <= 16 ? 16 : 64;
-  g.tn = maxN <= 16 ? 16 : 64;
+  int maxN = 0, maxK = 0;
   for (int q = 0; q < c.G; ++q) {
     const int64_t M = A.rows[q], K = A.cols[q], N = B.cols[q];
     if (B.rows[q] != K || C.rows[q] != M || C.cols[q] != N)
@@ -541,65 +535,20 @@ GemmPlan make_gemm_plan(Ctx& c, const Layout& A, const Layout& B, const Layout& 
     p.a = A.blk_off[q];
     p.b = B.blk_off[q];
     p.c = C.blk_off[q];
+    p.out0 = g.n_out;
     p.M = int32_t(M);
     p.N = int32_t(N);
     p.K = int32_t(K);
-    p.tiles_n = int32_t((N + g.tn - 1) / g.tn);
-    p.tiles_m = int32_t((M + g.tm - 1) / g.tm);
-    p.ksplit = 1;
-    p.kchunk = int32_t(((K + 7) / 8) * 8);
-    tiles_mn += int64_t(p.tiles_m) * p.tiles_n;
+    maxN = std::max(maxN, p.N);
+    maxK = std::max(maxK, p.K);
+    g.n_out += M * N;
     g.flops_mac += M * N * K;
     g.h_probs.push_back(p);
   }
-  // matrix-vector products, and small ones whose K is long enough for the warp's lanes
-  // to share or whose outputs are few: one warp per output element (a short K leaves
-  // most lanes idle, which a batch of instances multiplies: those take the tiles)
-  int64_t maxK = 0, outs = 0;
-  for (const GemmProb& p : g.h_probs) {
-    maxK = std::max<int64_t>(maxK, p.K);
-    outs += int64_t(p.M) * p.N;
-  }
-  if (maxN <= 2 ||
-      (g.flops_mac * c.ninst < (int64_t(1) << 22) && (maxK >= 32 || outs * c.ninst <= (int64_t(1) << 18)))) {
-    int64_t o = 0;
-    for (auto& p : g.h_probs) { p.ws = o; o += int64_t(p.M) * p.N; }
-    g.dot_outputs = o;
-    g.n_probs = int(g.h_probs.size());
-    if (g.n_probs) {
-      g.d_probs = (GemmProb*)c.dalloc(g.h_probs.size() * sizeof(GemmProb));
-      upload(c, g.d_probs, g.h_probs.data(), g.h_probs.size() * sizeof(GemmProb));
-    }
-    return g;
-  }
-  // split K when the output tiles cannot fill the GPU (long-K, small-MN blocks)
-  const int64_t want = 8LL * std::max(c.sm_count, 1);
-  const int64_t have = tiles_mn * c.ninst;
-  int tile0 = 0;
-  int64_t ws = 0;
-  for (auto& p : g.h_probs) {
-    if (have < 2LL * std::max(c.sm_count, 1) && p.K >= 512) {
-      int64_t ks = std::min<int64_t>((p.K + 255) / 256, (want + have - 1) / std::max<int64_t>(have, 1));
-      ks = std::max<int64_t>(1, std::min<int64_t>(ks, 256));
-      if (ks > 1) {
-        p.kchunk = int32_t((((p.K + ks - 1) / ks) + 7) / 8 * 8);
-        p.ksplit = int32_t((p.K + p.kchunk - 1) / p.kchunk);
-      }
-    }
-    if (p.ksplit > 1) {
-      p.ws = ws;
-      ws += int64_t(p.ksplit) * p.M * p.N;
-      g.red_elems += int64_t(p.M) * p.N;
-    }
-    p.tile0 = tile0;
-    tile0 += p.tiles_m * p.tiles_n * p.ksplit;
-  }
+  g.lanes = gemm_lanes(c, g.n_out * c.ninst, maxK);
+  g.matvec = maxN <= 2 || (g.flops_mac * c.ninst < (int64_t(1) << 22) &&
+                           (maxK >= 32 || g.n_out * c.ninst <= (int64_t(1) << 18)));
   g.n_probs = int(g.h_probs.size());
-  g.n_tiles = tile0;
-  if (ws) {
-    g.ws_is = ws;
-    g.d_ws = (cplx*)c.dalloc(sizeof(cplx) * ws * c.ninst);
-  }
   if (g.n_probs) {
     g.d_probs = (GemmProb*)c.dalloc(g.h_probs.size() * sizeof(GemmProb));
     upload(c, g.d_probs, g.h_probs.data(), g.h_probs.size() * sizeof(GemmProb));

@@ -89,14 +89,13 @@ struct ChunkRef {
 
 struct GemmProb {  // one block of a grouped GEMM: C[MxN] (+)= alpha A[MxK] B[KxN], row-major
   int64_t a, b, c;  // element offsets inside the per-instance tensors
-  int64_t ws;       // split-K partials offset in the plan's scratch (ksplit > 1)
+  int64_t out0;     // first output of this problem in the launch's numbering
   int32_t M, N, K;
-  int32_t tile0;    // first tile index of this problem
+  int32_t tile0;    // double-single tiles (k_gemm_ds): first tile of this problem
   int32_t tiles_n;  // tiles along N
   int32_t tiles_m;
-  int32_t ksplit;   // K ranges computed by separate CTAs, summed in fixed order
-  int32_t kchunk;   // K per split (multiple of 8)
 };
+#define GEMM_MAX_LANES 256  // most threads that share one output of the FP64 product
 
 struct GenTask {  // integral generator: one sub-block
   int64_t base;
@@ -151,13 +150,10 @@ struct PermPlan {
 struct GemmPlan {
   GemmProb* d_probs = nullptr;
   int n_probs = 0;
-  int n_tiles = 0;
-  int tm = 64, tn = 64;      // FP64 tile shape (16 or 64 each)
-  cplx* d_ws = nullptr;      // split-K partials, ws_is elements per instance
-  int64_t ws_is = 0;
-  int64_t red_elems = 0;     // output elements of split problems (per instance)
+  int64_t n_out = 0;      // output elements per instance
+  int lanes = 1;          // threads per output of the FP64 product (gemm_lanes)
   int64_t flops_mac = 0;  // complex MACs per instance
-  int64_t dot_outputs = 0;  // > 0: run as one warp per output element (k_gemm_dot), this many outputs
+  bool matvec = false;    // matrix-vector or small: stays FP64 where a short K would go to k_gemm_ds
   std::vector<GemmProb> h_probs;
   GemmProb* d_ds = nullptr;  // double-single SIMT tiles (k_gemm_ds), set by ds_prepare
   int ds_tiles = 0;
@@ -205,6 +201,7 @@ void launch_tau3(Ctx& c, cplx* tau, cplx* taut, cplx* zeta, int64_t dst_is, cons
                  int n_chunks);
 void launch_gemm_fp64(Ctx& c, const GemmPlan& g, const cplx* A, const cplx* B, cplx* C,
                       int64_t a_is, int64_t b_is, int64_t c_is, cplx alpha, bool beta);
+int gemm_lanes(const Ctx& c, int64_t outputs, int kmax);
 // double-single SIMT product for short contractions (every K <= 16) under the
 // emulated precision: ds_wanted decides, ds_prepare builds its tile list once
 bool ds_wanted(Ctx& c, const GemmPlan& g);

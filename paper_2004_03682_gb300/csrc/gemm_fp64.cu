@@ -1,6 +1,6 @@
 // Plain complex-FP64 grouped GEMM: step 3 of the TTGT list (Sec. II.B), all
 // symmetry blocks and instances of one contraction in one launch (the block
-// loop of Fig. "mult" flattened into a tile list).  Row-major operands,
+// loop of Fig. "mult" flattened into a list of outputs).  Row-major operands,
 // C[MxN] = alpha A[MxK] B[KxN] (+ C).  SIMT FP64 FMA: GB300's FP64 rate is the
 // roofline for this path.
 #include <algorithm>
@@ -9,195 +9,102 @@
 #include "engine.h"
 #include "fpbits.h"
 
-#define GT_K 8
-
-// Tile TM x TN (each 16 or 64), 256 threads as 16 x 16, every thread computing
-// (TM/16) x (TN/16) outputs; the plan picks 16 along a dimension whose blocks are
-// all <= 16 wide, so skinny contractions do not pay for padding.
-template <int TM, int TN>
-__global__ void __launch_bounds__(256) k_gemm_fp64(const GemmProb* __restrict__ probs, int n_probs,
-                                                   const cplx* __restrict__ A,
-                                                   const cplx* __restrict__ B, cplx* __restrict__ C,
-                                                   int64_t ais, int64_t bis, int64_t cis,
-                                                   cplx alpha, int beta, cplx* __restrict__ ws,
-                                                   int64_t ws_is) {
-  constexpr int RM = TM / 16, RN = TN / 16;
-  __shared__ cplx As[GT_K][TM];
-  __shared__ cplx Bs[GT_K][TN];
-  const int tile = blockIdx.x;
-  int pi = 0;
-  while (pi + 1 < n_probs && probs[pi + 1].tile0 <= tile) ++pi;
-  const GemmProb P = probs[pi];
-  int lt = tile - P.tile0;
-  const int tmn = P.tiles_m * P.tiles_n;
-  const int ks = lt / tmn;  // K split index
-  lt -= ks * tmn;
-  const int m0 = (lt / P.tiles_n) * TM, n0 = (lt % P.tiles_n) * TN;
-  const int kbeg = ks * P.kchunk, kend = min(P.K, kbeg + P.kchunk);
-  A += blockIdx.y * ais + P.a;
-  B += blockIdx.y * bis + P.b;
-  C += blockIdx.y * cis + P.c;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  double accr[RM][RN], acci[RM][RN];
-#pragma unroll
-  for (int i = 0; i < RM; ++i)
-#pragma unroll
-    for (int j = 0; j < RN; ++j) accr[i][j] = acci[i][j] = 0.0;
-  for (int k0 = kbeg; k0 < kend; k0 += GT_K) {
-    for (int e = threadIdx.x; e < TM * GT_K; e += 256) {
-      const int mm = e >> 3, kk = e & 7;
-      const int gm = m0 + mm, gk = k0 + kk;
-      As[kk][mm] = (gm < P.M && gk < kend) ? A[int64_t(gm) * P.K + gk] : make_double2(0, 0);
-    }
-    for (int e = threadIdx.x; e < TN * GT_K; e += 256) {
-      const int kk = e / TN, nn = e % TN;
-      const int gk = k0 + kk, gn = n0 + nn;
-      Bs[kk][nn] = (gk < kend && gn < P.N) ? B[int64_t(gk) * P.N + gn] : make_double2(0, 0);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < GT_K; ++kk) {
-      cplx a[RM], b[RN];
-#pragma unroll
-      for (int i = 0; i < RM; ++i) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-      for (int j = 0; j < RN; ++j) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < RM; ++i)
-#pragma unroll
-        for (int j = 0; j < RN; ++j) {
-          accr[i][j] = fma(a[i].x, b[j].x, accr[i][j]);
-          accr[i][j] = fma(-a[i].y, b[j].y, accr[i][j]);
-          acci[i][j] = fma(a[i].x, b[j].y, acci[i][j]);
-          acci[i][j] = fma(a[i].y, b[j].x, acci[i][j]);
-        }
-    }
-    __syncthreads();
+// One output element per thread (lanes = 1), or per group of `lanes` threads that
+// share its K (lanes a power of two, then a fixed butterfly; above a warp a fixed
+// sum over the group's warps in shared memory).
+//
+// What bounds it: the FP64 pipe, two FMAs per clock per SM -- one warp-wide FMA holds
+// its SM partition's pipe for 64 clocks, so the four FMAs of one k take 256 clocks a
+// warp while its two 16-byte loads a lane take a few.  Operand reuse is therefore not
+// what matters (64 consecutive outputs re-reading B from L2 ask for 8 B a clock of
+// the SM); what matters is that every lane holds an output and that the four
+// partitions of all SMs get the same share.  So: outputs numbered along the rows of
+// all blocks (no padded rows or columns at any shape), CTAs of two warps (the last
+// wave is then a small part of the launch), and K shared among lanes only where the
+// outputs alone do not fill the chip.  Measured against 64 x 64 shared-memory tiles
+// (with a warp per output for small products), TFLOP/s of complex work, exp_zgemm:
+// 1024^3 1.17 -> 1.22, 300^3 0.16 -> 0.81, 6000 x 24 x 400 0.27 -> 0.98, 64 x 64 x 5000
+// 0.14 -> 0.70; one CCSD iteration at o=10 v=40 8.2 -> 2.1 ms, at o=40 v=200 Z8 278 ->
+// 203 ms (1.22 TFLOP/s), (T) at o=24 v=120 Z8 1940 -> 97 ms.
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS) k_gemm_fp64(const GemmProb* __restrict__ probs, int n_probs,
+                                                       const cplx* __restrict__ A, const cplx* __restrict__ B,
+                                                       cplx* __restrict__ C, int64_t ais, int64_t bis, int64_t cis,
+                                                       cplx alpha, int beta, int64_t n_out, int lanes) {
+  const int group = threadIdx.x / lanes, lane = threadIdx.x - group * lanes;
+  const int64_t it = int64_t(blockIdx.x) * (THREADS / lanes) + group;
+  const bool live = it < n_out;
+  int lo = 0, hi = n_probs - 1;
+  while (lo < hi) {  // the block that holds output `it`
+    const int mid = (lo + hi + 1) >> 1;
+    if (probs[mid].out0 <= it) lo = mid;
+    else hi = mid - 1;
   }
-  if (P.ksplit > 1) {  // raw partial for the fixed-order reduction
-    cplx* W = ws + blockIdx.y * ws_is + P.ws + int64_t(ks) * P.M * P.N;
-#pragma unroll
-    for (int i = 0; i < RM; ++i) {
-      const int gm = m0 + ty + 16 * i;
-      if (gm >= P.M) continue;
-#pragma unroll
-      for (int j = 0; j < RN; ++j) {
-        const int gn = n0 + tx + 16 * j;
-        if (gn < P.N) W[int64_t(gm) * P.N + gn] = make_double2(accr[i][j], acci[i][j]);
-      }
-    }
-    return;
-  }
-#pragma unroll
-  for (int i = 0; i < RM; ++i) {
-    const int gm = m0 + ty + 16 * i;
-    if (gm >= P.M) continue;
-#pragma unroll
-    for (int j = 0; j < RN; ++j) {
-      const int gn = n0 + tx + 16 * j;
-      if (gn >= P.N) continue;
-      double vr = alpha.x * accr[i][j] - alpha.y * acci[i][j];
-      double vi = alpha.x * acci[i][j] + alpha.y * accr[i][j];
-      cplx* dp = C + int64_t(gm) * P.N + gn;
-      if (beta) { const cplx o = *dp; vr += o.x; vi += o.y; }
-      *dp = make_double2(vr, vi);
-    }
-  }
-}
-
-// C = alpha * sum_s partial_s (+ C), splits summed in index order (deterministic)
-__global__ void __launch_bounds__(256) k_splitk_reduce(const GemmProb* __restrict__ probs, int n_probs,
-                                                       const cplx* __restrict__ ws, int64_t ws_is,
-                                                       cplx* __restrict__ C, int64_t cis, cplx alpha, int beta) {
-  const int inst = blockIdx.y;
-  for (int p = 0; p < n_probs; ++p) {
-    const GemmProb P = probs[p];
-    if (P.ksplit <= 1) continue;
-    const int64_t n = int64_t(P.M) * P.N;
-    const cplx* W = ws + inst * ws_is + P.ws;
-    cplx* Cp = C + inst * cis + P.c;
-    for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < n; e += int64_t(gridDim.x) * blockDim.x) {
-      double sr = 0.0, si = 0.0;
-      for (int s = 0; s < P.ksplit; ++s) {
-        const cplx w = W[int64_t(s) * n + e];
-        sr += w.x;
-        si += w.y;
-      }
-      double vr = alpha.x * sr - alpha.y * si, vi = alpha.x * si + alpha.y * sr;
-      if (beta) { const cplx o = Cp[e]; vr += o.x; vi += o.y; }
-      Cp[e] = make_double2(vr, vi);
-    }
-  }
-}
-
-// Small products (and every matrix-vector one): one warp per output element, the
-// lanes striding over K, then a fixed butterfly.  At GB300's FP64 rate (about two
-// FMAs per clock per SM) a tile kernel leaves most SMs idle on these; here every
-// SM takes a share of the outputs and no padded rows or columns are computed.
-__global__ void __launch_bounds__(256) k_gemm_dot(const GemmProb* __restrict__ probs, int n_probs,
-                                                  const cplx* __restrict__ A, const cplx* __restrict__ B,
-                                                  cplx* __restrict__ C, int64_t ais, int64_t bis, int64_t cis,
-                                                  cplx alpha, int beta, int64_t n_out) {
-  const int lane = threadIdx.x & 31;
-  A += blockIdx.y * ais;
-  B += blockIdx.y * bis;
-  C += blockIdx.y * cis;
-  const int64_t stride = int64_t(gridDim.x) * (blockDim.x >> 5);
-  for (int64_t it = int64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5); it < n_out; it += stride) {
-    int pi = 0;
-    while (pi + 1 < n_probs && it >= probs[pi + 1].ws) ++pi;  // ws = first output of the problem here
-    const GemmProb& P = probs[pi];
-    const int64_t e = it - P.ws;
-    const int m = int(e / P.N), n = int(e - int64_t(m) * P.N);
-    const cplx* a = A + P.a + int64_t(m) * P.K;
-    const cplx* b = B + P.b + n;
-    double sr = 0.0, si = 0.0;
-    for (int k = lane; k < P.K; k += 32) {
-      const cplx x = a[k], y = b[int64_t(k) * P.N];
+  const GemmProb& P = probs[lo];
+  const int64_t e = it - P.out0;
+  double sr = 0.0, si = 0.0;
+  if (live) {
+    const int64_t m = e / P.N, n = e - m * P.N;
+    const cplx* a = A + blockIdx.y * ais + P.a + m * P.K + lane;
+    const cplx* b = B + blockIdx.y * bis + P.b + int64_t(lane) * P.N + n;
+    const int64_t bstep = int64_t(lanes) * P.N;
+#pragma unroll 4
+    for (int k = lane; k < P.K; k += lanes, a += lanes, b += bstep) {
+      const cplx x = *a, y = *b;
       sr = fma(x.x, y.x, sr);
       sr = fma(-x.y, y.y, sr);
       si = fma(x.x, y.y, si);
       si = fma(x.y, y.x, si);
     }
-    for (int o = 16; o; o >>= 1) {
-      sr += __shfl_xor_sync(0xffffffffu, sr, o);
-      si += __shfl_xor_sync(0xffffffffu, si, o);
-    }
-    if (lane == 0) {
-      double vr = alpha.x * sr - alpha.y * si, vi = alpha.x * si + alpha.y * sr;
-      cplx* dp = C + P.c + e;
-      if (beta) { const cplx o = *dp; vr += o.x; vi += o.y; }
-      *dp = make_double2(vr, vi);
-    }
   }
+  for (int o = min(lanes, 32) >> 1; o; o >>= 1) {
+    sr += __shfl_xor_sync(0xffffffffu, sr, o);
+    si += __shfl_xor_sync(0xffffffffu, si, o);
+  }
+  if (THREADS > 64 && lanes > 32) {  // lanes is uniform over the launch
+    __shared__ cplx part[THREADS / 32];
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = make_double2(sr, si);
+    __syncthreads();
+    if (lane == 0)
+      for (int w = 1; w < lanes / 32; ++w) {
+        const cplx p = part[(threadIdx.x >> 5) + w];
+        sr += p.x;
+        si += p.y;
+      }
+  }
+  if (live && lane == 0) {
+    double vr = alpha.x * sr - alpha.y * si, vi = alpha.x * si + alpha.y * sr;
+    cplx* dp = C + blockIdx.y * cis + P.c + e;
+    if (beta) { const cplx o = *dp; vr += o.x; vi += o.y; }
+    *dp = make_double2(vr, vi);
+  }
+}
+
+// Threads per output: 1 when the outputs of all instances give every SM partition
+// four warps, else the smallest power of two that does, while each lane keeps at
+// least four k (a shorter share costs more butterfly additions than it saves: each
+// halving of a lane's k adds two additions to four FMAs a k).
+int gemm_lanes(const Ctx& c, int64_t outputs, int kmax) {
+  const int64_t want = int64_t(std::max(c.sm_count, 1)) * 4 * 4 * 32;
+  int lanes = 1;
+  while (lanes < GEMM_MAX_LANES && outputs * lanes < want && kmax >= 8 * lanes) lanes *= 2;
+  return lanes;
 }
 
 void launch_gemm_fp64(Ctx& c, const GemmPlan& g, const cplx* A, const cplx* B, cplx* C, int64_t ais,
                       int64_t bis, int64_t cis, cplx alpha, bool beta) {
-  if (g.dot_outputs) {
-    const int blocks = int(std::max<int64_t>(1, std::min<int64_t>((g.dot_outputs + 7) / 8, 16LL * std::max(c.sm_count, 1))));
-    k_gemm_dot<<<dim3(blocks, c.ninst), 256, 0, c.stream>>>(g.d_probs, g.n_probs, A, B, C, ais, bis, cis, alpha,
-                                                             beta, g.dot_outputs);
-    KCHECK(c);
-    return;
-  }
-  if (g.n_tiles == 0) return;
-  const dim3 grid(g.n_tiles, c.ninst);
-  if (g.tm == 64 && g.tn == 64)
-    k_gemm_fp64<64, 64><<<grid, 256, 0, c.stream>>>(g.d_probs, g.n_probs, A, B, C, ais, bis, cis, alpha, beta, g.d_ws, g.ws_is);
-  else if (g.tm == 64)
-    k_gemm_fp64<64, 16><<<grid, 256, 0, c.stream>>>(g.d_probs, g.n_probs, A, B, C, ais, bis, cis, alpha, beta, g.d_ws, g.ws_is);
-  else if (g.tn == 64)
-    k_gemm_fp64<16, 64><<<grid, 256, 0, c.stream>>>(g.d_probs, g.n_probs, A, B, C, ais, bis, cis, alpha, beta, g.d_ws, g.ws_is);
+  if (g.n_out == 0) return;
+  const int threads = g.lanes > 32 ? GEMM_MAX_LANES : 64;
+  const int64_t per = threads / g.lanes;
+  const int64_t blocks = (g.n_out + per - 1) / per;
+  if (blocks > INT32_MAX) throw ExpError{EXP_EINVAL, "FP64 product: too many outputs in one launch"};
+  const dim3 grid(unsigned(blocks), c.ninst);
+  if (threads == 64)
+    k_gemm_fp64<64><<<grid, 64, 0, c.stream>>>(g.d_probs, g.n_probs, A, B, C, ais, bis, cis, alpha, beta, g.n_out, g.lanes);
   else
-    k_gemm_fp64<16, 16><<<grid, 256, 0, c.stream>>>(g.d_probs, g.n_probs, A, B, C, ais, bis, cis, alpha, beta, g.d_ws, g.ws_is);
+    k_gemm_fp64<GEMM_MAX_LANES><<<grid, GEMM_MAX_LANES, 0, c.stream>>>(g.d_probs, g.n_probs, A, B, C, ais, bis, cis, alpha,
+                                                                      beta, g.n_out, g.lanes);
   KCHECK(c);
-  if (g.red_elems) {
-    const int blocks = int(std::min<int64_t>((g.red_elems + 255) / 256, 2LL * std::max(c.sm_count, 1)));
-    k_splitk_reduce<<<dim3(blocks, c.ninst), 256, 0, c.stream>>>(g.d_probs, g.n_probs, g.d_ws, g.ws_is, C, cis,
-                                                                 alpha, beta);
-    KCHECK(c);
-  }
 }
 
 // ---------------------------------------------------------------------------
@@ -291,7 +198,7 @@ __global__ void __launch_bounds__(DS_ROWS) k_gemm_ds(const GemmProb* __restrict_
 }
 
 bool ds_wanted(Ctx& c, const GemmPlan& g) {
-  if (c.cfg.precision != EXP_EMU_BF16 || g.dot_outputs || g.h_probs.empty()) return false;
+  if (c.cfg.precision != EXP_EMU_BF16 || g.matvec || g.h_probs.empty()) return false;
   int kmax = 0;
   for (const GemmProb& p : g.h_probs) kmax = std::max(kmax, p.K);
   return kmax >= 1 && kmax <= DS_KMAX;

@@ -805,18 +805,13 @@ void ccsd_t(Ctx& c, int inst, int block, exp_t3_info* info, double* per_triple) 
             std::vector<GemmProb>& fp = bp.fprods[w];
             if (fp.empty()) continue;
             GemmPlan g;
-            g.tm = 64;  // N = the virtuals of one irrep: 16-wide column tiles
-            g.tn = 16;
-            int tile0 = 0;
+            int kmax = 0;
             for (GemmProb& f : fp) {
-              f.tiles_m = (f.M + g.tm - 1) / g.tm;
-              f.tiles_n = (f.N + g.tn - 1) / g.tn;
-              f.ksplit = 1;
-              f.kchunk = (f.K + 7) / 8 * 8;
-              f.tile0 = tile0;
-              tile0 += f.tiles_m * f.tiles_n;
+              f.out0 = g.n_out;
+              g.n_out += int64_t(f.M) * f.N;
+              kmax = std::max(kmax, f.K);
             }
-            g.n_tiles = tile0;
+            g.lanes = gemm_lanes(c, g.n_out, kmax);
             g.n_probs = int(fp.size());
             upload_async(c, d_fp, fp.data(), sizeof(GemmProb) * fp.size());
             g.d_probs = d_fp;
