@@ -4,12 +4,13 @@
 //     h1 = relu(W1 x + b1), h2 = relu(W2 h1 + b2), y = W3 h2 + b3,
 //     t2 = (1 + y0 + i y1) t_MP2,
 // trained on converged amplitudes of earlier solves (loss: mean |t2 - t2_conv|^2 /
-// 0.05^2, Adam).  Hand-written forward, backward and update kernels.  bf16 mode:
-// weights and activations rounded to BF16, and the three width-128 layer products
-// (h1 W2^T forward, gz2 W2 and gz2^T h1 backward, the gradients rounded to BF16 as
-// operands) on the tensor cores, mma m16n8k16 with FP32 accumulation; check mode:
-// plain FP32 on the SIMT pipes.  The paper has no counterpart; the guess only changes
-// the starting point of the amplitude iteration, never its fixed point.
+// 0.05^2, Adam).  Hand-written forward, backward and update kernels.  bf16 mode
+// (k_mlp_grad_bf, k_mlp_apply_bf): weights and activations rounded to BF16, and the
+// three width-128 layer products (h1 W2^T forward, gz2 W2 and gz2^T h1 backward, the
+// gradients rounded to BF16 as operands) on the tensor cores, mma m16n8k16 with FP32
+// accumulation; check mode (k_mlp_grad, k_mlp_apply): plain FP32 on the SIMT pipes.
+// The paper has no counterpart; the guess only changes the starting point of the
+// amplitude iteration, never its fixed point.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -27,39 +28,6 @@ constexpr int OFF_W1 = 0, OFF_B1 = OFF_W1 + W * NF, OFF_W2 = OFF_B1 + W, OFF_B2 
               OFF_W3 = OFF_B2 + W, OFF_B3 = OFF_W3 + NO * W, NPARAM = OFF_B3 + NO;
 constexpr int TS = 32;  // samples per CTA tile
 constexpr int MLP_SMEM = (2 * W * W + W * NF + 2 * W + NO * W + NO + 3 * TS * W + TS * NF + TS * NO) * 4 + 64;
-
-__device__ __forceinline__ float rb(float x, int bf) { return bf ? __bfloat162float(__float2bfloat16_rn(x)) : x; }
-
-// ---------------------------------------------------------------------------
-// The width-128 layer products in the bf16 mode run on the tensor cores: warp-level
-// mma.m16n8k16 with BF16 operands and FP32 accumulation.  Fragment layout (PTX ISA,
-// m16n8k16 .bf16; g = lane / 4, t = lane % 4): A registers {(g, 2t), (g + 8, 2t),
-// (g, 2t + 8), (g + 8, 2t + 8)} with the next column in the high half; B registers
-// {(2t, g), (2t + 8, g)} with the next row in the high half; D {(g, 2t), (g, 2t + 1),
-// (g + 8, 2t), (g + 8, 2t + 1)}.
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<const uint32_t*>(&v);
-}
-__device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
-// D[16 x 8] += A[r0 .. r0+16, k0 .. k0+16] B[k0 .. k0+16, c0 .. c0+8] for element accessors
-// A(r, k), B(k, c) (values already on the BF16 grid, or rounded here)
-template <typename FA, typename FB>
-__device__ __forceinline__ void mma_tile(float (&d)[4], int r0, int c0, int k0, FA A, FB B) {
-  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const uint32_t a[4] = {pack_bf16(A(r0 + g, k0 + 2 * t), A(r0 + g, k0 + 2 * t + 1)),
-                         pack_bf16(A(r0 + g + 8, k0 + 2 * t), A(r0 + g + 8, k0 + 2 * t + 1)),
-                         pack_bf16(A(r0 + g, k0 + 2 * t + 8), A(r0 + g, k0 + 2 * t + 9)),
-                         pack_bf16(A(r0 + g + 8, k0 + 2 * t + 8), A(r0 + g + 8, k0 + 2 * t + 9))};
-  const uint32_t b[2] = {pack_bf16(B(k0 + 2 * t, c0 + g), B(k0 + 2 * t + 1, c0 + g)),
-                         pack_bf16(B(k0 + 2 * t + 8, c0 + g), B(k0 + 2 * t + 9, c0 + g))};
-  mma_16816(d, a, b);
-}
 
 struct Smem {
   float* W2;   // [u][k]
@@ -93,58 +61,34 @@ __device__ Smem carve(float* base) {
   return m;
 }
 
-__device__ void load_params(const float* __restrict__ P, Smem& m, int bf) {
+__device__ void load_params(const float* __restrict__ P, Smem& m) {
   for (int e = threadIdx.x; e < W * W; e += blockDim.x) {
     const int u = e / W, k = e % W;
-    const float v = rb(P[OFF_W2 + e], bf);
+    const float v = P[OFF_W2 + e];
     m.W2[e] = v;
     m.W2T[k * W + u] = v;
   }
-  for (int e = threadIdx.x; e < W * NF; e += blockDim.x) m.W1[e] = rb(P[OFF_W1 + e], bf);
+  for (int e = threadIdx.x; e < W * NF; e += blockDim.x) m.W1[e] = P[OFF_W1 + e];
   for (int e = threadIdx.x; e < W; e += blockDim.x) { m.b1[e] = P[OFF_B1 + e]; m.b2[e] = P[OFF_B2 + e]; }
-  for (int e = threadIdx.x; e < NO * W; e += blockDim.x) m.W3[e] = rb(P[OFF_W3 + e], bf);
+  for (int e = threadIdx.x; e < NO * W; e += blockDim.x) m.W3[e] = P[OFF_W3 + e];
   if (threadIdx.x < NO) m.b3[threadIdx.x] = P[OFF_B3 + threadIdx.x];
 }
 
 // forward for the TS samples whose features sit in m.x (ns valid); y into m.gy
-__device__ void forward_tile(Smem& m, int ns, int bf) {
+__device__ void forward_tile(Smem& m, int ns) {
   for (int e = threadIdx.x; e < TS * W; e += blockDim.x) {
     const int s = e / W, u = e % W;
     float z = m.b1[u];
 #pragma unroll
     for (int f = 0; f < NF; ++f) z += m.W1[u * NF + f] * m.x[s * NF + f];
-    m.h1[e] = s < ns ? rb(fmaxf(z, 0.f), bf) : 0.f;
+    m.h1[e] = s < ns ? fmaxf(z, 0.f) : 0.f;
   }
   __syncthreads();
-  if (bf) {
-    // z2 = h1 W2^T on the tensor cores: warp w takes the 16 units 16w .. 16w + 15 of all
-    // TS = 32 samples (two 16-row by two 8-column tiles, K = 128 in steps of 16)
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    float d[2][2][4] = {};
-    auto A = [&](int r, int k) { return m.h1[r * W + k]; };
-    auto B = [&](int k, int c) { return m.W2[c * W + k]; };
-#pragma unroll
-    for (int k0 = 0; k0 < W; k0 += 16)
-#pragma unroll
-      for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-        for (int nt = 0; nt < 2; ++nt) mma_tile(d[mt][nt], 16 * mt, 16 * w + 8 * nt, k0, A, B);
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-      for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int s = 16 * mt + g + (q >> 1) * 8, u = 16 * w + 8 * nt + 2 * t + (q & 1);
-          m.h2[s * W + u] = s < ns ? rb(fmaxf(d[mt][nt][q] + m.b2[u], 0.f), bf) : 0.f;
-        }
-  } else {
-    for (int e = threadIdx.x; e < TS * W; e += blockDim.x) {
-      const int s = e / W, u = e % W;
-      float z = m.b2[u];
-      for (int k = 0; k < W; ++k) z += m.W2T[k * W + u] * m.h1[s * W + k];
-      m.h2[e] = s < ns ? rb(fmaxf(z, 0.f), bf) : 0.f;
-    }
+  for (int e = threadIdx.x; e < TS * W; e += blockDim.x) {
+    const int s = e / W, u = e % W;
+    float z = m.b2[u];
+    for (int k = 0; k < W; ++k) z += m.W2T[k * W + u] * m.h1[s * W + k];
+    m.h2[e] = s < ns ? fmaxf(z, 0.f) : 0.f;
   }
   __syncthreads();
   for (int e = threadIdx.x; e < TS * NO; e += blockDim.x) {
@@ -163,12 +107,12 @@ __device__ void forward_tile(Smem& m, int ns, int bf) {
 __global__ void __launch_bounds__(256) k_mlp_grad(const float* __restrict__ P, const float* __restrict__ X,
                                                   const float2* __restrict__ TM, const float2* __restrict__ TG,
                                                   const int* __restrict__ idx, int b0, int nb, float inv_n,
-                                                  float* __restrict__ grad, double* __restrict__ loss, int bf) {
+                                                  float* __restrict__ grad, double* __restrict__ loss) {
   extern __shared__ float sm[];
   Smem m = carve(sm);
   __shared__ float aW1[W * NF], ab1[W], ab2[W];
   __shared__ float lsum[TS];
-  load_params(P, m, bf);
+  load_params(P, m);
   float gW2[W * W / 256];  // entries threadIdx.x + 256 j
   float gW3 = 0.f, gb3 = 0.f;
 #pragma unroll
@@ -186,7 +130,7 @@ __global__ void __launch_bounds__(256) k_mlp_grad(const float* __restrict__ P, c
       m.x[e] = s < ns ? X[int64_t(idx[t0 + s]) * NF + e % NF] : 0.f;
     }
     __syncthreads();
-    forward_tile(m, ns, bf);
+    forward_tile(m, ns);
     if (threadIdx.x < TS) {
       const int s = threadIdx.x;
       float l = 0.f, g0 = 0.f, g1 = 0.f;
@@ -220,32 +164,12 @@ __global__ void __launch_bounds__(256) k_mlp_grad(const float* __restrict__ P, c
       m.g[e] = m.h2[e] > 0.f ? a : 0.f;
     }
     __syncthreads();
-    if (bf) {
-      // gW2 += gz2^T h1 on the tensor cores (gz2 rounded to BF16): warp w holds the 16 rows
-      // u = 16w .. 16w + 15 of all 128 columns, 16 column tiles x 4 entries per thread
-      const int w = threadIdx.x >> 5;
-      auto A = [&](int u, int sm_) { return m.g[sm_ * W + u]; };
-      auto B = [&](int sm_, int k) { return m.h1[sm_ * W + k]; };
 #pragma unroll
-      for (int k0 = 0; k0 < TS; k0 += 16)
-#pragma unroll
-        for (int nt = 0; nt < W / 8; ++nt) {
-          float* acc = gW2 + 4 * nt;
-          float d[4] = {acc[0], acc[1], acc[2], acc[3]};
-          mma_tile(d, 16 * w, 8 * nt, k0, A, B);
-          acc[0] = d[0];
-          acc[1] = d[1];
-          acc[2] = d[2];
-          acc[3] = d[3];
-        }
-    } else {
-#pragma unroll
-      for (int j = 0; j < W * W / 256; ++j) {
-        const int e = threadIdx.x + 256 * j, u = e / W, k = e % W;
-        float a = 0.f;
-        for (int s = 0; s < ns; ++s) a += m.g[s * W + u] * m.h1[s * W + k];
-        gW2[j] += a;
-      }
+    for (int j = 0; j < W * W / 256; ++j) {
+      const int e = threadIdx.x + 256 * j, u = e / W, k = e % W;
+      float a = 0.f;
+      for (int s = 0; s < ns; ++s) a += m.g[s * W + u] * m.h1[s * W + k];
+      gW2[j] += a;
     }
     if (threadIdx.x < W) {
       float a = 0.f;
@@ -253,33 +177,11 @@ __global__ void __launch_bounds__(256) k_mlp_grad(const float* __restrict__ P, c
       ab2[threadIdx.x] += a;
     }
     __syncthreads();
-    if (bf) {  // gz1 = (gz2 W2) . relu'(z1), over h2: on the tensor cores, warp w the columns 16w ..
-      const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-      float d[2][2][4] = {};
-      auto A = [&](int sm_, int u) { return m.g[sm_ * W + u]; };
-      auto B = [&](int u, int k) { return m.W2T[k * W + u]; };
-#pragma unroll
-      for (int k0 = 0; k0 < W; k0 += 16)
-#pragma unroll
-        for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-          for (int nt = 0; nt < 2; ++nt) mma_tile(d[mt][nt], 16 * mt, 16 * w + 8 * nt, k0, A, B);
-#pragma unroll
-      for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-        for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const int sm_ = 16 * mt + g + (q >> 1) * 8, k = 16 * w + 8 * nt + 2 * t + (q & 1);
-            m.h2[sm_ * W + k] = m.h1[sm_ * W + k] > 0.f ? d[mt][nt][q] : 0.f;
-          }
-    } else {
-      for (int e = threadIdx.x; e < TS * W; e += blockDim.x) {  // gz1 = (gz2 W2) . relu'(z1), over h2
-        const int s = e / W, k = e % W;
-        float a = 0.f;
-        for (int u = 0; u < W; ++u) a += m.g[s * W + u] * m.W2[u * W + k];
-        m.h2[e] = m.h1[e] > 0.f ? a : 0.f;
-      }
+    for (int e = threadIdx.x; e < TS * W; e += blockDim.x) {  // gz1 = (gz2 W2) . relu'(z1), over h2
+      const int s = e / W, k = e % W;
+      float a = 0.f;
+      for (int u = 0; u < W; ++u) a += m.g[s * W + u] * m.W2[u * W + k];
+      m.h2[e] = m.h1[e] > 0.f ? a : 0.f;
     }
     __syncthreads();
     for (int e = threadIdx.x; e < W * NF; e += blockDim.x) {
@@ -295,19 +197,8 @@ __global__ void __launch_bounds__(256) k_mlp_grad(const float* __restrict__ P, c
     }
   }
   __syncthreads();
-  if (bf) {  // gW2 fragments: warp w rows 16w + g (+8), column tile nt, columns 2t (+1)
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
 #pragma unroll
-    for (int nt = 0; nt < W / 8; ++nt)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int u = 16 * w + g + (q >> 1) * 8, k = 8 * nt + 2 * t + (q & 1);
-        atomicAdd(&grad[OFF_W2 + u * W + k], gW2[4 * nt + q]);
-      }
-  } else {
-#pragma unroll
-    for (int j = 0; j < W * W / 256; ++j) atomicAdd(&grad[OFF_W2 + threadIdx.x + 256 * j], gW2[j]);
-  }
+  for (int j = 0; j < W * W / 256; ++j) atomicAdd(&grad[OFF_W2 + threadIdx.x + 256 * j], gW2[j]);
   atomicAdd(&grad[OFF_W3 + threadIdx.x], gW3);
   if (threadIdx.x < NO) atomicAdd(&grad[OFF_B3 + threadIdx.x], gb3);
   for (int e = threadIdx.x; e < W * NF; e += blockDim.x) atomicAdd(&grad[OFF_W1 + e], aW1[e]);
@@ -331,24 +222,28 @@ __global__ void k_adam(float* __restrict__ P, const float* __restrict__ G, float
   P[k] -= lr * mh / (sqrtf(vh) + eps);
 }
 
-// features of element p of instance inst from <ab||ij> (Vd), D and the instance's max |V|
-__device__ __forceinline__ void elem_features(cplx v, double d, float vmax, float* x, float2* tm) {
-  const double ar = v.x / d, ai = v.y / d;
-  *tm = make_float2(float(ar), float(ai));
-  x[0] = float(hypot(ar, ai) / 0.05);
-  x[1] = float(-d / 10.0);
-  x[2] = vmax > 0.f ? float(hypot(v.x, v.y)) / vmax : 0.f;
+// First-order amplitude and features of one element from <ab||ij>, D and the instance's
+// max |V|.  FP64 instructions are the cost (GB300 issues two a clock and SM): one square
+// root serves |t| and |V| = |t| |D|.
+__device__ __forceinline__ cplx elem_features(cplx v, double d, float vmax, float* x) {
+  const cplx t = make_double2(v.x / d, v.y / d);
+  const double ta = sqrt(t.x * t.x + t.y * t.y);  // (over- and underflow only beyond the FP32 range)
+  x[0] = float(ta * 20.0);
+  x[1] = float(d * -0.1);
+  x[2] = vmax > 0.f ? float(ta * fabs(d)) / vmax : 0.f;
+  return t;
 }
 
 __global__ void k_vmax(const cplx* __restrict__ V, int64_t vis, int64_t n2, float* __restrict__ vmax) {
   const int inst = blockIdx.y;
-  float m = 0.f;
+  unsigned long long q = 0;  // bits of the largest |V|^2: non-negative doubles order as their bits
   for (int64_t k = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; k < n2; k += int64_t(gridDim.x) * blockDim.x) {
     const cplx v = V[inst * vis + k];
-    m = fmaxf(m, float(hypot(v.x, v.y)));
+    q = max(q, (unsigned long long)__double_as_longlong(fma(v.x, v.x, v.y * v.y)));
   }
-  for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) atomicMax((int*)&vmax[inst], __float_as_int(m));  // m >= 0: int order = float order
+  for (int o = 16; o; o >>= 1) q = max(q, __shfl_xor_sync(0xffffffffu, q, o));
+  if ((threadIdx.x & 31) == 0)  // >= 0: int order = float order
+    atomicMax((int*)&vmax[inst], __float_as_int(float(sqrt(__longlong_as_double((long long)q)))));
 }
 
 // training samples from the unique elements (a<b, i<j, no ghost) of converged instances
@@ -362,10 +257,9 @@ __global__ void k_extract(const cplx* __restrict__ V, int64_t vis, const double*
     const int64_t p = elems[k];
     const int64_t o = base + int64_t(ii) * ne + k;
     float x[NF];
-    float2 tm;
-    elem_features(V[inst * vis + p], D[inst * namp + n1 + p], vmax[inst], x, &tm);
+    const cplx tm = elem_features(V[inst * vis + p], D[inst * namp + n1 + p], vmax[inst], x);
     for (int f = 0; f < NF; ++f) X[o * NF + f] = x[f];
-    TM[o] = tm;
+    TM[o] = make_float2(float(tm.x), float(tm.y));
     const cplx t = T[inst * namp + n1 + p];
     TG[o] = make_float2(float(t.x), float(t.y));
   }
@@ -374,24 +268,23 @@ __global__ void k_extract(const cplx* __restrict__ V, int64_t vis, const double*
 // inference over every t2 element of every instance: t2 = (1 + y0 + i y1) <ab||ij> / D
 __global__ void __launch_bounds__(256) k_mlp_apply(const float* __restrict__ P, const cplx* __restrict__ V, int64_t vis,
                                                    const double* __restrict__ D, cplx* __restrict__ T, int64_t namp,
-                                                   int64_t n1, int64_t n2, const float* __restrict__ vmax, int bf) {
+                                                   int64_t n1, int64_t n2, const float* __restrict__ vmax) {
   extern __shared__ float sm[];
   Smem m = carve(sm);
-  load_params(P, m, bf);
+  load_params(P, m);
   const int inst = blockIdx.y;
   __syncthreads();
   for (int64_t t0 = int64_t(blockIdx.x) * TS; t0 < n2; t0 += int64_t(gridDim.x) * TS) {
     const int ns = int(n2 - t0 < TS ? n2 - t0 : TS);
     for (int e = threadIdx.x; e < TS; e += blockDim.x) {
       if (e < ns) {
-        float2 tm;
-        elem_features(V[inst * vis + t0 + e], D[inst * namp + n1 + t0 + e], vmax[inst], &m.x[e * NF], &tm);
+        elem_features(V[inst * vis + t0 + e], D[inst * namp + n1 + t0 + e], vmax[inst], &m.x[e * NF]);
       } else {
         for (int f = 0; f < NF; ++f) m.x[e * NF + f] = 0.f;
       }
     }
     __syncthreads();
-    forward_tile(m, ns, bf);
+    forward_tile(m, ns);
     for (int s = threadIdx.x; s < ns; s += blockDim.x) {
       const cplx v = V[inst * vis + t0 + s];
       const double d = D[inst * namp + n1 + t0 + s];
@@ -400,6 +293,390 @@ __global__ void __launch_bounds__(256) k_mlp_apply(const float* __restrict__ P, 
       T[inst * namp + n1 + t0 + s] = make_double2(mr * ar - mi * ai, mr * ai + mi * ar);
     }
     __syncthreads();
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The bf16 mode.  Fragment layout of mma m16n8k16 .bf16 (PTX ISA; g = lane / 4, t = lane
+// % 4): A registers {(g, 2t), (g + 8, 2t), (g, 2t + 8), (g + 8, 2t + 8)} with the next
+// column in the high half; B registers {(2t, g), (2t + 8, g)} with the next row in the high
+// half; D {(g, 2t), (g, 2t + 1), (g + 8, 2t), (g + 8, 2t + 1)}.  So two neighbouring D
+// column tiles, packed to BF16, are one A fragment of the next product, and a warp takes
+// its samples through layers 1 and 2 in registers: layer 1 (three inputs) is computed
+// straight into A fragments.  Layer 3 (two outputs) reads h2 back from shared memory, a
+// whole row per lane, which sums y over the units in their order.
+//
+// What bounds it: instruction issue (the mma's with their operand loads and the FP32 layers
+// about equally), then FP64 for the features.  The first
+// form kept FP32 activations in shared memory, gathered every fragment element by element
+// (12 loads and 6 conversions per mma) and gave the two-output layer to 64 of 256 threads:
+// o=10 v=40, one guess of 64 instances (10.2 million elements): 28.6 -> 1.8 ms; one pass over
+// 561,600 training samples in batches of 65,536: 2.52 -> 0.56 ms.
+constexpr int LDB = W + 8;       // BF16 row stride in shared memory: 272 B, rows 16 B apart in the banks
+constexpr int GT = 128;          // samples per group of the gradient: 16 per warp, four tiles of TS
+constexpr int LDG = W + 4;       // FP32 row stride of gz1
+constexpr int BF_THREADS = 256;
+constexpr int BF_APPLY = 128;  // threads of the inference CTA: 3 of them an SM at up to 170 registers
+constexpr int BF_PARAMS = W * 16 + W * 8 + W * 4;      // per unit: (W1 row, b1), W3 column, b2
+constexpr int BF_FWD_SMEM = W * LDB * 2 + BF_PARAMS;   // + W2
+constexpr int BF_APPLY_SMEM = BF_FWD_SMEM + BF_APPLY * LDB * 2;  // + h2
+constexpr int BF_GRAD_SMEM = BF_FWD_SMEM + 3 * GT * LDB * 2 + GT * LDG * 4 + GT * 16 + GT * 8;
+
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+__device__ __forceinline__ float bf_lo(uint32_t v) { return __uint_as_float(v << 16); }
+__device__ __forceinline__ float bf_hi(uint32_t v) { return __uint_as_float(v & 0xFFFF0000u); }
+__device__ __forceinline__ float bf_round(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
+__device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t* a, uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// four 8 x 8 BF16 matrices; lane l gives the address of row l % 8 of matrix l / 8
+template <bool TRANS>
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const __nv_bfloat16* p) {
+  const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+  if (TRANS)
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+  else
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+}
+
+struct BfParams {
+  __nv_bfloat16* W2;  // [u][k], stride LDB
+  float4* in;         // [u]: W1[u][0..2], b1[u]
+  float2* W3;         // [u]: W3[0][u], W3[1][u]
+  float* b2;          // [u]
+};
+__device__ BfParams bf_load(const float* __restrict__ P, uint8_t* base) {
+  BfParams p;
+  p.W2 = (__nv_bfloat16*)base;
+  p.in = (float4*)(base + W * LDB * 2);
+  p.W3 = (float2*)(p.in + W);
+  p.b2 = (float*)(p.W3 + W);
+  for (int e = threadIdx.x; e < W * W; e += blockDim.x)
+    p.W2[(e / W) * LDB + e % W] = __float2bfloat16_rn(P[OFF_W2 + e]);
+  for (int u = threadIdx.x; u < W; u += blockDim.x) {
+    p.in[u] = make_float4(bf_round(P[OFF_W1 + u * NF]), bf_round(P[OFF_W1 + u * NF + 1]), bf_round(P[OFF_W1 + u * NF + 2]),
+                          P[OFF_B1 + u]);
+    p.W3[u] = make_float2(bf_round(P[OFF_W3 + u]), bf_round(P[OFF_W3 + W + u]));
+    p.b2[u] = P[OFF_B2 + u];
+  }
+  return p;
+}
+
+// h1 = relu(W1 x + b1) of the warp's 16 samples as the A fragments of layer 2; x0, x1: the
+// features of rows g and g + 8
+__device__ __forceinline__ void bf_layer1(const BfParams& p, const float (&x0)[NF], const float (&x1)[NF],
+                                          uint32_t (&a)[8][4]) {
+  const int t = threadIdx.x & 3;
+#pragma unroll
+  for (int ks = 0; ks < 8; ++ks)
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      const float4 u = p.in[16 * ks + 8 * half + 2 * t], w = p.in[16 * ks + 8 * half + 2 * t + 1];
+      auto z = [](const float4& q, const float (&x)[NF]) {
+        return fmaxf(q.w + q.x * x[0] + q.y * x[1] + q.z * x[2], 0.f);
+      };
+      a[ks][2 * half] = pack_bf16(z(u, x0), z(w, x0));
+      a[ks][2 * half + 1] = pack_bf16(z(u, x1), z(w, x1));
+    }
+}
+
+// Layer 2 of MT groups of 16 samples: h2 = relu(z2) rounded, to rows 16 mt + g (+ 8) of
+// sh (row stride LDB).
+template <int MT>
+__device__ __forceinline__ void bf_layer2(const BfParams& p, const uint32_t (&a)[MT][8][4], __nv_bfloat16* sh) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  // B[k][u] = W2[u][k]: matrices (u 0-7, k 0-7), (u 0-7, k 8-15), (u 8-15, k 0-7), (u 8-15, k 8-15)
+  const __nv_bfloat16* wb = p.W2 + ((lane >> 4) * 8 + (lane & 7)) * LDB + ((lane >> 3) & 1) * 8;
+#pragma unroll 2
+  for (int n2 = 0; n2 < 8; ++n2) {  // 16 units at a time
+    float d[MT][2][4] = {};
+#pragma unroll
+    for (int ks = 0; ks < 8; ++ks) {
+      uint32_t b[4];
+      ldsm4<false>(b, wb + 16 * n2 * LDB + 16 * ks);
+#pragma unroll
+      for (int mt = 0; mt < MT; ++mt) {
+        mma_16816(d[mt][0], a[mt][ks], b[0], b[1]);
+        mma_16816(d[mt][1], a[mt][ks], b[2], b[3]);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const float2 c = *reinterpret_cast<const float2*>(p.b2 + 16 * n2 + 8 * q + 2 * t);
+#pragma unroll
+      for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+          *reinterpret_cast<uint32_t*>(sh + (16 * mt + g + 8 * r) * LDB + 16 * n2 + 8 * q + 2 * t) =
+              pack_bf16(fmaxf(d[mt][q][2 * r] + c.x, 0.f), fmaxf(d[mt][q][2 * r + 1] + c.y, 0.f));
+    }
+  }
+}
+
+// Gradient of the batch loss, bf16 mode.  A CTA walks tiles of TS samples (grid-stride),
+// four at a time, a warp 16 samples: forward, loss, gz2 = (gy W3) . relu'(z2) and gz1 =
+// (gz2 W2) . relu'(z1) in its own registers, then h1, h2, gz2 (BF16) and gz1 (FP32) of the
+// group meet in shared memory for the sums over samples: gW2 = gz2^T h1 on the tensor
+// cores (warp w the 16 rows u = 16w.., kept in registers over all tiles), the others in
+// FP32, one chain per thread in sample order (a sum per tile for W1, b1 and b2, one running
+// sum for W3 and b3).  One atomicAdd per entry and CTA at the end.
+__global__ void __launch_bounds__(BF_THREADS, 1)
+    k_mlp_grad_bf(const float* __restrict__ P, const float* __restrict__ X, const float2* __restrict__ TM,
+                  const float2* __restrict__ TG, const int* __restrict__ idx, int b0, int nb, float inv_n,
+                  float* __restrict__ grad, double* __restrict__ loss) {
+  extern __shared__ __align__(16) uint8_t bsm[];
+  const BfParams p = bf_load(P, bsm);
+  __syncthreads();
+  __nv_bfloat16* sh1 = (__nv_bfloat16*)(bsm + BF_FWD_SMEM);  // [s][k]
+  __nv_bfloat16* sh2 = sh1 + GT * LDB;                       // [s][u]
+  __nv_bfloat16* sg2 = sh2 + GT * LDB;                       // [s][u]
+  float* sg1 = (float*)(sg2 + GT * LDB);                     // [s][k]
+  float4* sx = (float4*)(sg1 + GT * LDG);                    // [s] features
+  float2* sgy = (float2*)(sx + GT);                          // [s] dL/dy
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  float gW2[16][4] = {};
+  const int cu = threadIdx.x & (W - 1), co = threadIdx.x / W;  // sums over samples: unit, output
+  const float2 w3 = p.W3[cu];
+  float cW3 = 0.f, cb3 = 0.f, cb2 = 0.f, cb1 = 0.f, cW1[NF] = {};
+  double lacc = 0.0;
+  const int ntile = (nb + TS - 1) / TS;
+  for (int tile0 = blockIdx.x; tile0 < ntile; tile0 += 4 * gridDim.x) {
+    // 16-sample piece w of the group: half w % 2 of tile tile0 + (w / 2) gridDim; the live
+    // pieces are the first np
+    auto first = [&](int w) { return (tile0 + (w >> 1) * int(gridDim.x)) * TS + 16 * (w & 1); };
+    int np = 0;
+    while (np < GT / 16 && first(np) < nb) ++np;
+    const int t0 = first(warp);  // the warp's first sample in the batch
+    if (warp < np) {
+      // lane l < 16 reads sample l of the warp's
+      float4 xs = make_float4(0.f, 0.f, 0.f, 0.f);
+      float2 tm = make_float2(0.f, 0.f), tg = tm;
+      if (lane < 16 && t0 + lane < nb) {
+        const int64_t k = idx[b0 + t0 + lane];
+        xs = make_float4(X[k * NF], X[k * NF + 1], X[k * NF + 2], 0.f);
+        tm = TM[k];
+        tg = TG[k];
+      }
+      if (lane < 16) sx[16 * warp + lane] = xs;
+      float xr[2][NF];
+      float2 tmr[2], tgr[2];
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        xr[r][0] = __shfl_sync(0xffffffffu, xs.x, g + 8 * r);
+        xr[r][1] = __shfl_sync(0xffffffffu, xs.y, g + 8 * r);
+        xr[r][2] = __shfl_sync(0xffffffffu, xs.z, g + 8 * r);
+        tmr[r] = make_float2(__shfl_sync(0xffffffffu, tm.x, g + 8 * r), __shfl_sync(0xffffffffu, tm.y, g + 8 * r));
+        tgr[r] = make_float2(__shfl_sync(0xffffffffu, tg.x, g + 8 * r), __shfl_sync(0xffffffffu, tg.y, g + 8 * r));
+      }
+      uint32_t a[1][8][4];
+      bf_layer1(p, xr[0], xr[1], a[0]);
+      bf_layer2<1>(p, a, sh2 + 16 * warp * LDB);
+      __syncwarp();
+      // layer 3: lane = (sample, output)
+      float y;
+      {
+        const int o = lane >> 4;
+        const __nv_bfloat16* h = sh2 + (16 * warp + (lane & 15)) * LDB;
+        const float* wo = reinterpret_cast<const float*>(p.W3) + o;
+        y = P[OFF_B3 + o];
+#pragma unroll 4
+        for (int k = 0; k < W; k += 8) {
+          const uint4 q = *reinterpret_cast<const uint4*>(h + k);
+          const uint32_t v[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            y += wo[2 * (k + 2 * j)] * bf_lo(v[j]);
+            y += wo[2 * (k + 2 * j + 1)] * bf_hi(v[j]);
+          }
+        }
+      }
+      // loss and dL/dy of rows g and g + 8 (zero past the batch)
+      float gy[2][NO];
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const float mr = 1.f + __shfl_sync(0xffffffffu, y, g + 8 * r), mi = __shfl_sync(0xffffffffu, y, 16 + g + 8 * r);
+        const float rr = mr * tmr[r].x - mi * tmr[r].y - tgr[r].x, ri = mr * tmr[r].y + mi * tmr[r].x - tgr[r].y;
+        const float c = 2.f * inv_n / (0.05f * 0.05f);
+        const bool live = t0 + g + 8 * r < nb;
+        gy[r][0] = live ? c * (rr * tmr[r].x + ri * tmr[r].y) : 0.f;   // Re(conj(r) tmp2)
+        gy[r][1] = live ? c * (-rr * tmr[r].y + ri * tmr[r].x) : 0.f;  // Re(conj(r) i tmp2)
+        if (t == 0) {
+          if (live) lacc += double((rr * rr + ri * ri) / (0.05f * 0.05f));
+          sgy[16 * warp + g + 8 * r] = make_float2(gy[r][0], gy[r][1]);
+        }
+      }
+      // gz2, packed as the A fragments of gz2 W2, and h1, gz2 into shared memory
+      uint32_t ga[8][4];
+#pragma unroll
+      for (int nt = 0; nt < 16; ++nt) {
+        const float2 u = p.W3[8 * nt + 2 * t], w = p.W3[8 * nt + 2 * t + 1];
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          const int at = (16 * warp + g + 8 * r) * LDB + 8 * nt + 2 * t;
+          const uint32_t h = *reinterpret_cast<const uint32_t*>(sh2 + at);
+          const float q0 = __fmaf_rn(gy[r][1], u.y, __fmul_rn(gy[r][0], u.x));
+          const float q1 = __fmaf_rn(gy[r][1], w.y, __fmul_rn(gy[r][0], w.x));
+          const uint32_t v = pack_bf16((h & 0xFFFFu) ? q0 : 0.f, (h >> 16) ? q1 : 0.f);
+          ga[nt >> 1][(nt & 1) * 2 + r] = v;
+          *reinterpret_cast<uint32_t*>(sh1 + at) = a[0][nt >> 1][(nt & 1) * 2 + r];
+          *reinterpret_cast<uint32_t*>(sg2 + at) = v;
+        }
+      }
+      // gz1: B[u][k] = W2[u][k] through transposed loads, 16 columns k at a time
+      const __nv_bfloat16* wt = p.W2 + (((lane >> 3) & 1) * 8 + (lane & 7)) * LDB + (lane >> 4) * 8;
+#pragma unroll
+      for (int n2 = 0; n2 < 8; ++n2) {
+        float d[2][4] = {};
+#pragma unroll
+        for (int ks = 0; ks < 8; ++ks) {
+          uint32_t b[4];
+          ldsm4<true>(b, wt + 16 * ks * LDB + 16 * n2);
+          mma_16816(d[0], ga[ks], b[0], b[1]);
+          mma_16816(d[1], ga[ks], b[2], b[3]);
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+#pragma unroll
+          for (int r = 0; r < 2; ++r) {
+            const uint32_t h = a[0][n2][2 * q + r];  // h1 at the same place: relu'(z1)
+            *reinterpret_cast<float2*>(sg1 + (16 * warp + g + 8 * r) * LDG + 16 * n2 + 8 * q + 2 * t) =
+                make_float2((h & 0xFFFFu) ? d[q][2 * r] : 0.f, (h >> 16) ? d[q][2 * r + 1] : 0.f);
+          }
+      }
+    }
+    __syncthreads();
+    // gW2 += gz2^T h1 over the group's samples
+    {
+      const __nv_bfloat16* pa = sg2 + ((lane >> 4) * 8 + (lane & 7)) * LDB + 16 * warp + ((lane >> 3) & 1) * 8;
+      const __nv_bfloat16* pb = sh1 + (((lane >> 3) & 1) * 8 + (lane & 7)) * LDB + (lane >> 4) * 8;
+#pragma unroll 2
+      for (int ks = 0; ks < np; ++ks) {
+        uint32_t am[4];
+        ldsm4<true>(am, pa + 16 * ks * LDB);
+#pragma unroll
+        for (int n2 = 0; n2 < 8; ++n2) {
+          uint32_t b[4];
+          ldsm4<true>(b, pb + 16 * ks * LDB + 16 * n2);
+          mma_16816(gW2[2 * n2], am, b[0], b[1]);
+          mma_16816(gW2[2 * n2 + 1], am, b[2], b[3]);
+        }
+      }
+    }
+    // sums over the samples, a tile at a time
+    for (int s0 = 0; s0 < 16 * np; s0 += TS) {
+      const int s1 = min(s0 + TS, 16 * np);
+      if (co == 0) {  // W3[0], b2, b3[0]
+        float a = 0.f;
+#pragma unroll 8
+        for (int s = s0; s < s1; ++s) {
+          const float2 q = sgy[s];
+          const float h = __bfloat162float(sh2[s * LDB + cu]);
+          cW3 = __fmaf_rn(q.x, h, cW3);
+          cb3 += q.x;
+          a += h > 0.f ? __fmaf_rn(q.y, w3.y, __fmul_rn(q.x, w3.x)) : 0.f;
+        }
+        cb2 += a;
+      } else {  // W3[1], b3[1], W1, b1
+        float a = 0.f, a1[NF] = {};
+#pragma unroll 8
+        for (int s = s0; s < s1; ++s) {
+          const float q = sgy[s].y;
+          cW3 = __fmaf_rn(q, __bfloat162float(sh2[s * LDB + cu]), cW3);
+          cb3 += q;
+          const float z = sg1[s * LDG + cu];
+          const float4 x = sx[s];
+          a += z;
+          a1[0] = __fmaf_rn(z, x.x, a1[0]);
+          a1[1] = __fmaf_rn(z, x.y, a1[1]);
+          a1[2] = __fmaf_rn(z, x.z, a1[2]);
+        }
+        cb1 += a;
+#pragma unroll
+        for (int f = 0; f < NF; ++f) cW1[f] += a1[f];
+      }
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int nt = 0; nt < 16; ++nt)
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+      atomicAdd(reinterpret_cast<float2*>(&grad[OFF_W2 + (16 * warp + g + 8 * r) * W + 8 * nt + 2 * t]),
+                make_float2(gW2[nt][2 * r], gW2[nt][2 * r + 1]));
+  atomicAdd(&grad[OFF_W3 + threadIdx.x], cW3);
+  if (cu == 0) atomicAdd(&grad[OFF_B3 + co], cb3);
+  if (co == 0) {
+    atomicAdd(&grad[OFF_B2 + cu], cb2);
+  } else {
+    atomicAdd(&grad[OFF_B1 + cu], cb1);
+#pragma unroll
+    for (int f = 0; f < NF; ++f) atomicAdd(&grad[OFF_W1 + cu * NF + f], cW1[f]);
+  }
+  for (int o = 16; o; o >>= 1) lacc += __shfl_xor_sync(0xffffffffu, lacc, o);
+  if (lane == 0) atomicAdd(loss, lacc * inv_n);
+}
+
+// Inference, bf16 mode: 32 elements per warp step, one per lane for the features, layer 3
+// and the result, two 16-row groups for layer 2 (each W2 fragment load serves both).
+__global__ void __launch_bounds__(BF_APPLY, 3) k_mlp_apply_bf(const float* __restrict__ P, const cplx* __restrict__ V,
+                                                              int64_t vis, const double* __restrict__ D,
+                                                              cplx* __restrict__ T, int64_t namp, int64_t n1, int64_t n2,
+                                                              const float* __restrict__ vmax) {
+  extern __shared__ __align__(16) uint8_t bsm[];
+  const BfParams p = bf_load(P, bsm);
+  __syncthreads();
+  const int inst = blockIdx.y, lane = threadIdx.x & 31, g = lane >> 2;
+  __nv_bfloat16* sh = (__nv_bfloat16*)(bsm + BF_FWD_SMEM) + (threadIdx.x & ~31) * LDB;  // the warp's h2
+  const float vm = vmax[inst];
+  const cplx* v = V + inst * vis;
+  const double* d = D + inst * namp + n1;
+  cplx* out = T + inst * namp + n1;
+  const int64_t step = int64_t(gridDim.x) * BF_APPLY;
+  for (int64_t w0 = int64_t(blockIdx.x) * BF_APPLY + (threadIdx.x & ~31); w0 < n2; w0 += step) {
+    const int64_t e = w0 + lane;
+    float x[NF] = {0.f, 0.f, 0.f};
+    cplx tm = make_double2(0.0, 0.0);
+    if (e < n2) tm = elem_features(v[e], d[e], vm, x);
+    uint32_t a[2][8][4];
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt) {
+      float x0[NF], x1[NF];
+#pragma unroll
+      for (int f = 0; f < NF; ++f) {
+        x0[f] = __shfl_sync(0xffffffffu, x[f], 16 * mt + g);
+        x1[f] = __shfl_sync(0xffffffffu, x[f], 16 * mt + g + 8);
+      }
+      bf_layer1(p, x0, x1, a[mt]);
+    }
+    bf_layer2<2>(p, a, sh);
+    __syncwarp();
+    float y0 = P[OFF_B3], y1 = P[OFF_B3 + 1];
+#pragma unroll 4
+    for (int k = 0; k < W; k += 8) {
+      const uint4 q = *reinterpret_cast<const uint4*>(sh + lane * LDB + k);
+      const uint32_t h[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float4 w = *reinterpret_cast<const float4*>(p.W3 + k + 2 * j);
+        y0 += w.x * bf_lo(h[j]);
+        y1 += w.y * bf_lo(h[j]);
+        y0 += w.z * bf_hi(h[j]);
+        y1 += w.w * bf_hi(h[j]);
+      }
+    }
+    __syncwarp();
+    if (e < n2) {
+      const double mr = 1.0 + y0, mi = y1;
+      out[e] = make_double2(mr * tm.x - mi * tm.y, mr * tm.y + mi * tm.x);
+    }
   }
 }
 
@@ -489,6 +766,8 @@ extern "C" exp_status exp_mlp_create(const exp_allocator* alloc, void* stream, u
   CK(cudaGetLastError());
   CK(cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, MLP_SMEM));
   CK(cudaFuncSetAttribute(k_mlp_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, MLP_SMEM));
+  CK(cudaFuncSetAttribute(k_mlp_grad_bf, cudaFuncAttributeMaxDynamicSharedMemorySize, BF_GRAD_SMEM));
+  CK(cudaFuncSetAttribute(k_mlp_apply_bf, cudaFuncAttributeMaxDynamicSharedMemorySize, BF_APPLY_SMEM));
   CK(cudaStreamSynchronize(m->stream));
   *out = m;
   return EXP_OK;
@@ -614,8 +893,13 @@ static void grad_batch(exp_mlp* m, const float* X, const float2* TM, const float
                        int64_t nb) {
   CK(cudaMemsetAsync(m->G, 0, sizeof(float) * NPARAM, m->stream));
   const int blocks = int(std::min<int64_t>((nb + TS - 1) / TS, 304));
-  k_mlp_grad<<<blocks, 256, MLP_SMEM, m->stream>>>(m->P, X, TM, TG, idx, int(b0), int(nb), 1.f / float(nb), m->G,
-                                                   m->d_loss, m->bf);
+  if (m->bf) {
+    k_mlp_grad_bf<<<blocks, BF_THREADS, BF_GRAD_SMEM, m->stream>>>(m->P, X, TM, TG, idx, int(b0), int(nb), 1.f / float(nb),
+                                                                   m->G, m->d_loss);
+  } else {
+    k_mlp_grad<<<blocks, 256, MLP_SMEM, m->stream>>>(m->P, X, TM, TG, idx, int(b0), int(nb), 1.f / float(nb), m->G,
+                                                     m->d_loss);
+  }
   CK(cudaGetLastError());
 }
 
@@ -712,9 +996,18 @@ extern "C" exp_status exp_mlp_apply(exp_mlp* m, exp_ctx* x) {
   CK(cudaStreamSynchronize(m->stream));
   float* vm = ctx_vmax(m, c);
   const Tensor* Vd = ccsd_driver_integral(c);
-  const int blocks = int(std::max<int64_t>(1, std::min<int64_t>((c.n2 + TS - 1) / TS, 2 * 304)));
-  k_mlp_apply<<<dim3(blocks, c.ninst), 256, MLP_SMEM, c.stream>>>(m->P, Vd->d, Vd->is, c.d_D, c.d_T, c.namp, c.n1,
-                                                                   c.n2, vm, m->bf);
+  if (m->bf) {
+    // three CTAs an SM are resident; eight waves' worth over all instances, each keeping its
+    // parameters for many elements
+    const int64_t most = std::max<int64_t>(1, (8 * 3 * 152 + c.ninst - 1) / c.ninst);
+    const int blocks = int(std::max<int64_t>(1, std::min<int64_t>((c.n2 + BF_APPLY - 1) / BF_APPLY, most)));
+    k_mlp_apply_bf<<<dim3(blocks, c.ninst), BF_APPLY, BF_APPLY_SMEM, c.stream>>>(m->P, Vd->d, Vd->is, c.d_D, c.d_T, c.namp,
+                                                                                 c.n1, c.n2, vm);
+  } else {
+    const int blocks = int(std::max<int64_t>(1, std::min<int64_t>((c.n2 + TS - 1) / TS, 2 * 304)));
+    k_mlp_apply<<<dim3(blocks, c.ninst), 256, MLP_SMEM, c.stream>>>(m->P, Vd->d, Vd->is, c.d_D, c.d_T, c.namp, c.n1, c.n2,
+                                                                    vm);
+  }
   CK(cudaGetLastError());
   k_zero_t1<<<dim3(std::max<int64_t>(1, std::min<int64_t>((c.n1 + 255) / 256, 64)), c.ninst), 256, 0, c.stream>>>(
       c.d_T, c.namp, c.n1);
