@@ -805,13 +805,12 @@ void ccsd_t(Ctx& c, int inst, int block, exp_t3_info* info, double* per_triple) 
             std::vector<GemmProb>& fp = bp.fprods[w];
             if (fp.empty()) continue;
             GemmPlan g;
-            int kmax = 0;
+            // one thread per output whatever the batch holds: the order of each sum, and so
+            // every bit, is then the same for all block sizes
             for (GemmProb& f : fp) {
               f.out0 = g.n_out;
               g.n_out += int64_t(f.M) * f.N;
-              kmax = std::max(kmax, f.K);
             }
-            g.lanes = gemm_lanes(c, g.n_out, kmax);
             g.n_probs = int(fp.size());
             upload_async(c, d_fp, fp.data(), sizeof(GemmProb) * fp.size());
             g.d_probs = d_fp;
