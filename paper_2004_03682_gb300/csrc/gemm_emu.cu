@@ -48,13 +48,19 @@ constexpr int EMU_GM = 8;      // default row tiles per group of the GEMM work o
 #define ALPHA_POS_BIAS 64
 #define ALPHA_NEG_BIAS 64
 
-template <int S>
+// Real output columns per tile: as many as fit 256 TMEM columns.  Wider tiles copy fewer
+// bytes and issue fewer MMAs per output (an MMA of N columns takes N / 2 clocks, but about
+// 45 at least).  4096^3, 64 columns against 48: three slices 3.83 -> 2.96 ms, four 4.37 ->
+// 3.48 ms.
+constexpr int bn_of(int S) { return S <= 4 ? 64 : S == 5 ? 48 : 32; }
+
+template <int S, int COLS = bn_of(S)>
 struct Shape {
-  static constexpr int BN = S <= 5 ? 48 : 32;  // real output columns per tile
+  static constexpr int BN = COLS;
   // epilogue: WPQ warps on each TMEM lane quarter, each HW = BN / WPQ real columns of
   // every diagonal (more warps per tile shorten the per-warp chain of TMEM loads and
   // integer folds that bounds short-K products); warps 0 and 1 load and issue MMAs
-  static constexpr int WPQ = BN == 32 ? 4 : 3;
+  static constexpr int WPQ = BN == 48 ? 3 : 4;
   static constexpr int EPI = 4 * WPQ;
   static constexpr int HW = BN / WPQ;
   static constexpr int THREADS = 64 + 32 * EPI;
@@ -277,15 +283,15 @@ __device__ __forceinline__ EmuWork emu_work(const EmuProb* probs, int nprobs, in
 // The stage ring and the two TMEM accumulator buffers run on across items, so
 // the epilogue of one tile overlaps the MMAs of the next and the producer
 // prefetches across tile boundaries.
-template <int S>
-__global__ void __launch_bounds__(Shape<S>::THREADS, 1)
+template <int S, int COLS = bn_of(S)>
+__global__ void __launch_bounds__(Shape<S, COLS>::THREADS, 1)
     k_emu_gemm(const EmuProb* probs, int nprobs, int n_tiles, int n_work, int gm,
                const __nv_bfloat16* __restrict__ Asl, const __nv_bfloat16* __restrict__ Bsl,
                const int* __restrict__ Aex, const int* __restrict__ Bex, cplx* __restrict__ C, int64_t asl_is,
                int64_t bsl_is, int64_t aex_is, int64_t bex_is, int64_t c_is, cplx alpha, int alpha_e, int beta,
                int* __restrict__ gerr, cplx* __restrict__ ws, int64_t ws_is, EmuWaitTest wt,
                const int* __restrict__ t2p) {
-  using SH = Shape<S>;
+  using SH = Shape<S, COLS>;
   constexpr int STAGES = SH::STAGES;
   const unsigned long long wns = wt.wait_ns;
   // test hook (-1 = off): CTA 0 never issues the copies of its k-block skip_g, so the
@@ -451,10 +457,9 @@ __global__ void __launch_bounds__(Shape<S>::THREADS, 1)
       // first output column of this warp
       const int j0 = cpx ? W.nt * (SH::BN / 2) + h * (HW / 2) : W.nt * SH::BN + h * HW;
       const int ei = gi < P.M ? Aex[W.inst * aex_is + P.a_ex + gi] : 0;
-      int fj[HW / 2];  // complex columns' exponents (real columns load theirs at the store)
-#pragma unroll
-      for (int jj = 0; jj < HW / 2; ++jj)
-        fj[jj] = (cpx && gi < P.M && j0 + jj < P.N) ? Bex[W.inst * bex_is + P.b_ex + j0 + jj] : 0;
+      // the exponent of output column j0 + lane, handed out by shuffle (with 16 epilogue warps
+      // of 16 columns a register per column would spill)
+      const int fjl = (lane < (cpx ? HW / 2 : HW) && j0 + lane < P.N) ? Bex[W.inst * bex_is + P.b_ex + j0 + lane] : 0;
       for (int ch = 0; ch < nchunks; ++ch, ++gc) {
         const int buf = gc & 1;
         if (!mbar_wait(&accf[buf], (gc >> 1) & 1, abort, gerr, wns)) { ok = false; break; }
@@ -488,21 +493,22 @@ __global__ void __launch_bounds__(Shape<S>::THREADS, 1)
         if (lane == 0) mbar_arrive(&acce[buf]);
       }
       if (!ok) break;
-      if (gi >= P.M) continue;
+      if (nv8 == 0) continue;  // no outputs in this warp
+      const bool live = gi < P.M;
       if (!cpx) {  // real operands: column u of the warp is output column j0 + u, imaginary part 0
         if (P.ksplit > 1) {
           longlong2* Wp = reinterpret_cast<longlong2*>(ws + W.inst * ws_is + P.ws) + int64_t(W.ks) * P.M * P.N +
                           int64_t(gi) * P.N;
 #pragma unroll
           for (int u = 0; u < HW; ++u)
-            if (j0 + u < P.N) Wp[j0 + u] = make_longlong2(R[u], 0ll);
+            if (live && j0 + u < P.N) Wp[j0 + u] = make_longlong2(R[u], 0ll);
         } else {
           cplx* Crow = C + W.inst * c_is + P.c_off + int64_t(gi) * P.N;
 #pragma unroll
           for (int u = 0; u < HW; ++u) {
             const int gj = j0 + u;
-            if (gj < P.N) {
-              const int e = ei + Bex[W.inst * bex_is + P.b_ex + gj] - BETA * (S + 1);
+            const int e = ei + __shfl_sync(0xffffffffu, fjl, u) - BETA * (S + 1);
+            if (live && gj < P.N) {
               double vr, vi;
               if (alpha_e != ALPHA_GENERAL) {
                 const int k = alpha_e < 0 ? -alpha_e - ALPHA_NEG_BIAS : alpha_e - ALPHA_POS_BIAS;
@@ -526,15 +532,15 @@ __global__ void __launch_bounds__(Shape<S>::THREADS, 1)
 #pragma unroll
         for (int jj = 0; jj < HW / 2; ++jj) {
           const int gj = j0 + jj;
-          if (gj < P.N) Wp[gj] = make_longlong2(R[2 * jj], R[2 * jj + 1]);
+          if (live && gj < P.N) Wp[gj] = make_longlong2(R[2 * jj], R[2 * jj + 1]);
         }
       } else {
         cplx* Crow = C + W.inst * c_is + P.c_off + int64_t(gi) * P.N;
 #pragma unroll
         for (int jj = 0; jj < HW / 2; ++jj) {
           const int gj = j0 + jj;
-          if (gj < P.N) {
-            const int e = ei + fj[jj] - BETA * (S + 1);
+          const int e = ei + __shfl_sync(0xffffffffu, fjl, jj) - BETA * (S + 1);
+          if (live && gj < P.N) {
             double vr, vi;
             if (alpha_e != ALPHA_GENERAL) {  // alpha = +-2^k: folded into the exponent and sign
               const long long rr = alpha_e < 0 ? -R[2 * jj] : R[2 * jj], ri = alpha_e < 0 ? -R[2 * jj + 1] : R[2 * jj + 1];
@@ -786,16 +792,15 @@ __global__ void __launch_bounds__(256) k_split_a(const EmuProb* __restrict__ pro
 // one K range.  Work item = (column tile nt, 32-wide range kbh of the half); unit =
 // (column j, 8-group), lanes along j so the strided column reads coalesce; grid-stride
 // over all units.
-template <int S>
+template <int S, int COLS = bn_of(S)>
 __global__ void __launch_bounds__(256) k_split_b(const EmuProb* __restrict__ probs, int nprobs, int64_t total,
                                                  const cplx* __restrict__ B, int64_t b_is, const int* __restrict__ ex,
                                                  int64_t ex_is, __nv_bfloat16* __restrict__ out, int64_t out_is) {
-  using SH = Shape<S>;
   const int inst = blockIdx.y;
   for (int64_t U = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; U < total; U += int64_t(gridDim.x) * blockDim.x) {
     const int pi = prob_of_unit<UNIT_B>(probs, nprobs, U);
     const EmuProb& P = probs[pi];
-    const int NJ = ocols_of(P, SH::BN);   // output columns per tile
+    const int NJ = ocols_of(P, COLS);   // output columns per tile
     const int nj = P.brows / P.nh;  // stored columns per tile (NJ unless compact); nh B rows a column
     const int UB = nj * (KB / 8);
     const int64_t lu = U - P.bu0;
@@ -1045,8 +1050,6 @@ static void set_smem_attr() {
     done = true;
   }
 }
-
-static int bn_of(int S) { return S <= 5 ? 48 : 32; }
 
 bool emu_major_site(const std::string& site) {
   // the particle-particle ladder, X_amij (its t1 companion over <am||ef>), the two ring products
@@ -1707,8 +1710,10 @@ int64_t carve(int64_t& off, int64_t bytes) {
 template <int S>
 exp_status noalloc_launch(cudaStream_t st, unsigned char* base, int M, int N, int K, const cplx* A, const cplx* B,
                           cplx* Cout, cplx alpha, int beta, int sms, std::string& err) {
-  using SH = Shape<S>;
-  const int BN = SH::BN;
+  // three and four slices keep tiles of 48 columns here: wider ones would change which
+  // problems fit the fixed scratch
+  constexpr int BN = std::min(bn_of(S), 48);
+  using SH = Shape<S, BN>;
   EmuProb e{};
   e.M = M;
   e.N = N;
@@ -1785,14 +1790,14 @@ exp_status noalloc_launch(cudaStream_t st, unsigned char* base, int M, int N, in
   const int64_t nb = int64_t(e.tiles_n) * nkh_of(e) * (e.brows / 2) * (KB / 8);
   k_split_a<S, false><<<dim3(split_blocks(na, sms), 1), 256, 0, st>>>(d_probs, 1, na, A, 0, aex, 0, asl, 0);
   if (!launched("k_split_a")) return EXP_ECUDA;
-  k_split_b<S><<<dim3(split_blocks(nb, sms), 1), 256, 0, st>>>(d_probs, 1, nb, B, 0, bex, 0, bsl, 0);
+  k_split_b<S, BN><<<dim3(split_blocks(nb, sms), 1), 256, 0, st>>>(d_probs, 1, nb, B, 0, bex, 0, bsl, 0);
   if (!launched("k_split_b")) return EXP_ECUDA;
-  if (cudaFuncSetAttribute(k_emu_gemm<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, SH::SMEM) != cudaSuccess) {
+  if (cudaFuncSetAttribute(k_emu_gemm<S, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, SH::SMEM) != cudaSuccess) {
     err = "exp_zgemm_emu_noalloc: shared-memory attribute refused";
     return EXP_ECUDA;
   }
   const int n_work = int(tiles_mn * e.ksplit);
-  k_emu_gemm<S><<<dim3(unsigned(std::min(n_work, sms)), 1), SH::THREADS, SH::SMEM, st>>>(
+  k_emu_gemm<S, BN><<<dim3(unsigned(std::min(n_work, sms)), 1), SH::THREADS, SH::SMEM, st>>>(
       d_probs, 1, n_work, n_work, EMU_GM, asl, bsl, aex, bex, Cout, 0, 0, 0, 0, 0, alpha,
       e.ksplit > 1 ? ALPHA_GENERAL : alpha_code(alpha), beta, d_err, ws, 0, EmuWaitTest{2000000000ull, -1, 0}, nullptr);
   if (!launched("k_emu_gemm")) return EXP_ECUDA;
