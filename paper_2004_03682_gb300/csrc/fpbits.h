@@ -62,6 +62,29 @@ __device__ __forceinline__ float2 ds_split(double x) {
   return make_float2(h, __uint_as_float(lb ^ sgn));
 }
 
+// R 2^e in double-single: h is R rounded to 24 bits (nearest, ties to even), l the rest.
+// |R 2^e| < 2^-126 is flushed to zero, as ds_split does.
+__device__ __forceinline__ float2 ds_of_i64(long long R, int e) {
+  const unsigned sgn = unsigned((unsigned long long)R >> 32) & 0x80000000u;
+  unsigned long long m = R < 0 ? 0ull - (unsigned long long)R : (unsigned long long)R;
+  const int lz = __clzll((long long)m) & 63;
+  m <<= lz;  // leading one at bit 63 (R = 0: none): |R| 2^e = m 2^(e - lz)
+  unsigned hm = unsigned(m >> 40);
+  const unsigned long long rem = m & 0xFFFFFFFFFFull;
+  hm += rem + (hm & 1u) > (1ull << 39) ? 1u : 0u;
+  const long long r = (long long)(m - ((unsigned long long)hm << 40));  // the rest, |r| <= 2^39
+  const int fe = 190 + e - lz;  // biased exponent of hm 2^(40 + e - lz), hm in [2^23, 2^24]
+  // beyond the range of FP32: infinite, as the conversion gives
+  const int fc = fe < 255 ? fe : 255;
+  // a significand rounded up to 2^24 carries into the exponent field
+  const float h = __uint_as_float(sgn | ((unsigned(fc) << 23) + (fc == 255 ? 0u : hm - 0x800000u)));
+  const unsigned lb = __float_as_uint(__int2float_rn(int(r >> 9)));  // l = this 2^(9 + e - lz)
+  const int le = int((lb >> 23) & 0xFF) + 9 + e - lz;
+  const float l = __uint_as_float(((lb & 0x807FFFFFu) | (unsigned(le) << 23)) ^ sgn);
+  const bool tiny = fe < 1 || R == 0;
+  return make_float2(tiny ? 0.f : h, tiny || fc == 255 || le < 1 || (r < 512 && r >= 0) ? 0.f : l);
+}
+
 // signed integer significand and exponent of a float: f = m 2^e
 __device__ __forceinline__ void f32_parts(float f, int& m, int& e) {
   const unsigned u = __float_as_uint(f);

@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(Shape<S, COLS>::THREADS, 1)
                const int* __restrict__ Aex, const int* __restrict__ Bex, cplx* __restrict__ C, int64_t asl_is,
                int64_t bsl_is, int64_t aex_is, int64_t bex_is, int64_t c_is, cplx alpha, int alpha_e, int beta,
                int* __restrict__ gerr, cplx* __restrict__ ws, int64_t ws_is, EmuWaitTest wt,
-               const int* __restrict__ t2p) {
+               const int* __restrict__ t2p, int ds_out) {
   using SH = Shape<S, COLS>;
   constexpr int STAGES = SH::STAGES;
   const unsigned long long wns = wt.wait_ns;
@@ -495,6 +495,7 @@ __global__ void __launch_bounds__(Shape<S, COLS>::THREADS, 1)
       if (!ok) break;
       if (nv8 == 0) continue;  // no outputs in this warp
       const bool live = gi < P.M;
+      const int alpha_k = alpha_e < 0 ? -alpha_e - ALPHA_NEG_BIAS : alpha_e - ALPHA_POS_BIAS;  // alpha = +-2^alpha_k
       if (!cpx) {  // real operands: column u of the warp is output column j0 + u, imaginary part 0
         if (P.ksplit > 1) {
           longlong2* Wp = reinterpret_cast<longlong2*>(ws + W.inst * ws_is + P.ws) + int64_t(W.ks) * P.M * P.N +
@@ -509,10 +510,14 @@ __global__ void __launch_bounds__(Shape<S, COLS>::THREADS, 1)
             const int gj = j0 + u;
             const int e = ei + __shfl_sync(0xffffffffu, fjl, u) - BETA * (S + 1);
             if (live && gj < P.N) {
+              if (ds_out) {
+                const float2 x = ds_of_i64(alpha_e < 0 ? -R[u] : R[u], e + alpha_k);
+                reinterpret_cast<float4*>(Crow)[gj] = make_float4(x.x, x.y, 0.f, 0.f);
+                continue;
+              }
               double vr, vi;
               if (alpha_e != ALPHA_GENERAL) {
-                const int k = alpha_e < 0 ? -alpha_e - ALPHA_NEG_BIAS : alpha_e - ALPHA_POS_BIAS;
-                vr = scaled_i64(alpha_e < 0 ? -R[u] : R[u], e + k);
+                vr = scaled_i64(alpha_e < 0 ? -R[u] : R[u], e + alpha_k);
                 vi = 0.0;
               } else {
                 const double re = scaled_i64(R[u], e);
@@ -541,12 +546,17 @@ __global__ void __launch_bounds__(Shape<S, COLS>::THREADS, 1)
           const int gj = j0 + jj;
           const int e = ei + __shfl_sync(0xffffffffu, fjl, jj) - BETA * (S + 1);
           if (live && gj < P.N) {
+            if (ds_out) {
+              const float2 x = ds_of_i64(alpha_e < 0 ? -R[2 * jj] : R[2 * jj], e + alpha_k);
+              const float2 y = ds_of_i64(alpha_e < 0 ? -R[2 * jj + 1] : R[2 * jj + 1], e + alpha_k);
+              reinterpret_cast<float4*>(Crow)[gj] = make_float4(x.x, x.y, y.x, y.y);
+              continue;
+            }
             double vr, vi;
             if (alpha_e != ALPHA_GENERAL) {  // alpha = +-2^k: folded into the exponent and sign
               const long long rr = alpha_e < 0 ? -R[2 * jj] : R[2 * jj], ri = alpha_e < 0 ? -R[2 * jj + 1] : R[2 * jj + 1];
-              const int k = alpha_e < 0 ? -alpha_e - ALPHA_NEG_BIAS : alpha_e - ALPHA_POS_BIAS;
-              vr = scaled_i64(rr, e + k);
-              vi = scaled_i64(ri, e + k);
+              vr = scaled_i64(rr, e + alpha_k);
+              vi = scaled_i64(ri, e + alpha_k);
             } else {
               const double re = scaled_i64(R[2 * jj], e), im = scaled_i64(R[2 * jj + 1], e);
               vr = alpha.x * re - alpha.y * im;
@@ -1233,7 +1243,7 @@ static void launch_product(Ctx& c, EmuPlan* p, cplx* C, int64_t cis, cplx alpha,
                   c.stream>>>(
       p->d, np, p->n_tiles, n_work, p->gm, p->asl, p->bsl, p->aex, p->bex, C, p->asl_is, p->bsl_is, p->aex_is,
       p->bex_is, cis, alpha, p->red_elems ? ALPHA_GENERAL : alpha_code(alpha), beta ? 1 : 0, p->d_err, p->d_ws, p->ws_is,
-      emu_wait_test(), nullptr);
+      emu_wait_test(), nullptr, 0);
   KCHECK(c);
   if (reduce && p->red_elems) {
     int mks = 1;
@@ -1543,17 +1553,17 @@ void emu_set_slice(Ctx& c, EmuSet* s, const std::vector<EmuSetMat>& mats, const 
 
 template <int S>
 static void set_multiply_s(Ctx& c, const EmuProb* d, int np, int n_tiles, const EmuSet* A, const EmuSet* B, cplx* C,
-                           cplx alpha, int* gerr, const int* t2p) {
+                           int alpha_k, bool ds_out, int* gerr, const int* t2p) {
   set_smem_attr<S>();
   k_emu_gemm<S><<<dim3(std::min(n_tiles, std::max(c.sm_count, 1))), Shape<S>::THREADS, Shape<S>::SMEM,
                   c.stream>>>(
-      d, np, n_tiles, n_tiles, EMU_GM, A->sl, B->sl, A->ex, B->ex, C, 0, 0, 0, 0, 0, alpha, alpha_code(alpha), 0, gerr,
-      nullptr, 0, emu_wait_test(), t2p);
+      d, np, n_tiles, n_tiles, EMU_GM, A->sl, B->sl, A->ex, B->ex, C, 0, 0, 0, 0, 0, make_double2(1.0, 0.0),
+      alpha_k + ALPHA_POS_BIAS, 0, gerr, nullptr, 0, emu_wait_test(), t2p, ds_out ? 1 : 0);
   KCHECK(c);
 }
 
 void emu_set_multiply(Ctx& c, const EmuSet* A, const EmuSet* B, const std::vector<EmuSetProd>& prods, cplx* C,
-                      cplx alpha) {
+                      int alpha_k, bool ds_out) {
   if (A->b_side || !B->b_side || A->S != B->S || A->nh != B->nh)
     throw ExpError{EXP_EINVAL, "emulated product: operand sets do not match"};
   const int S = A->S;
@@ -1644,10 +1654,10 @@ void emu_set_multiply(Ctx& c, const EmuSet* A, const EmuSet* B, const std::vecto
     t2p = st->set_t2p;
   }
   switch (S) {
-    case 3: set_multiply_s<3>(c, st->set_d, np, nt, A, B, C, alpha, st->d_err, t2p); break;
-    case 4: set_multiply_s<4>(c, st->set_d, np, nt, A, B, C, alpha, st->d_err, t2p); break;
-    case 5: set_multiply_s<5>(c, st->set_d, np, nt, A, B, C, alpha, st->d_err, t2p); break;
-    default: set_multiply_s<6>(c, st->set_d, np, nt, A, B, C, alpha, st->d_err, t2p); break;
+    case 3: set_multiply_s<3>(c, st->set_d, np, nt, A, B, C, alpha_k, ds_out, st->d_err, t2p); break;
+    case 4: set_multiply_s<4>(c, st->set_d, np, nt, A, B, C, alpha_k, ds_out, st->d_err, t2p); break;
+    case 5: set_multiply_s<5>(c, st->set_d, np, nt, A, B, C, alpha_k, ds_out, st->d_err, t2p); break;
+    default: set_multiply_s<6>(c, st->set_d, np, nt, A, B, C, alpha_k, ds_out, st->d_err, t2p); break;
   }
 }
 
@@ -1799,7 +1809,7 @@ exp_status noalloc_launch(cudaStream_t st, unsigned char* base, int M, int N, in
   const int n_work = int(tiles_mn * e.ksplit);
   k_emu_gemm<S, BN><<<dim3(unsigned(std::min(n_work, sms)), 1), SH::THREADS, SH::SMEM, st>>>(
       d_probs, 1, n_work, n_work, EMU_GM, asl, bsl, aex, bex, Cout, 0, 0, 0, 0, 0, alpha,
-      e.ksplit > 1 ? ALPHA_GENERAL : alpha_code(alpha), beta, d_err, ws, 0, EmuWaitTest{2000000000ull, -1, 0}, nullptr);
+      e.ksplit > 1 ? ALPHA_GENERAL : alpha_code(alpha), beta, d_err, ws, 0, EmuWaitTest{2000000000ull, -1, 0}, nullptr, 0);
   if (!launched("k_emu_gemm")) return EXP_ECUDA;
   if (e.ksplit > 1) {
     launch_emu_reduce(d_probs, 1, e.ksplit, ws, 0, Cout, 0, aex, 0, bex, 0, S, alpha, beta, int64_t(M) * N, 1, sms, st);

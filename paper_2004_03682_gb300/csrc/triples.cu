@@ -58,6 +58,7 @@
 namespace {
 
 constexpr int T3_THREADS = 256;
+constexpr int T3_SEV = 512;  // split orbital energies a CTA of the energy kernel keeps
 
 // ---------------------------------------------------------------------------
 // Index tables of one context (irrep-sorted local indices; global spinor index =
@@ -227,11 +228,37 @@ __device__ __forceinline__ float2 ds_rcp(float2 a) {
   const float2 e = ds_add(make_float2(1.f, 0.f), ds_neg(q));
   return ds_add(make_float2(r, 0.f), ds_mul(make_float2(r, 0.f), e));
 }
-__device__ __forceinline__ dsc dsc_of(cplx z) { return dsc{ds_split(z.x), ds_split(z.y)}; }
+__device__ __forceinline__ dsc dsc_of(float4 z) { return dsc{make_float2(z.x, z.y), make_float2(z.z, z.w)}; }
 __device__ __forceinline__ dsc dsc_add(dsc a, dsc b) { return dsc{ds_add(a.re, b.re), ds_add(a.im, b.im)}; }
 __device__ __forceinline__ dsc dsc_sub(dsc a, dsc b) { return dsc{ds_add(a.re, ds_neg(b.re)), ds_add(a.im, ds_neg(b.im))}; }
 __device__ __forceinline__ dsc dsc_mul(dsc a, dsc b) {
   return dsc{ds_add(ds_mul(a.re, b.re), ds_neg(ds_mul(a.im, b.im))), ds_add(ds_mul(a.re, b.im), ds_mul(a.im, b.re))};
+}
+
+// Element of Y, t1 and <bc||jk> as the energy kernel reads them: double-single (re.h, re.l,
+// im.h, im.l) in the emulated precision, split once -- by the product's epilogue and by
+// k_t3_ds -- else FP64.  Splitting FP64 numbers at every use (six for the three Y elements,
+// four for each t1 V term, one for an orbital energy) was about half of the instructions
+// of k_t3_energy, which issue slots bound: o=40 v=200 Z8 71.3 -> 36.4 ms, o=18 v=72 Z4
+// 1.27 -> 0.45 ms, the product's epilogue unchanged.
+template <bool DS>
+struct T3ElemOf {
+  typedef cplx type;
+};
+template <>
+struct T3ElemOf<true> {
+  typedef float4 type;
+};
+template <bool DS>
+using T3Elem = typename T3ElemOf<DS>::type;
+
+// x (n complex numbers) in FP64 -> double-single, in place
+__global__ void __launch_bounds__(T3_THREADS) k_t3_ds(cplx* __restrict__ x, int64_t n) {
+  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
+    const cplx z = x[i];
+    const float2 re = ds_split(z.x), im = ds_split(z.y);
+    reinterpret_cast<float4*>(x)[i] = make_float4(re.x, re.y, im.x, im.y);
+  }
 }
 
 // Energy of one triple i<j<k and one pair irrep h of (b, c) per CTA: the sum over
@@ -242,8 +269,10 @@ __device__ __forceinline__ dsc dsc_mul(dsc a, dsc b) {
 // FP64 throughout.  Output: e3h[idx G + h].
 template <bool DS>
 __global__ void __launch_bounds__(T3_THREADS, 3) k_t3_energy(const T3Tri* __restrict__ tris, T3Tables T,
-                                                          const cplx* __restrict__ Yt, const int64_t* __restrict__ yoff,
-                                                          const cplx* __restrict__ t1, const cplx* __restrict__ V,
+                                                          const T3Elem<DS>* __restrict__ Yt,
+                                                          const int64_t* __restrict__ yoff,
+                                                          const T3Elem<DS>* __restrict__ t1,
+                                                          const T3Elem<DS>* __restrict__ V,
                                                           const double* __restrict__ eps, int o, int v,
                                                           cplx* __restrict__ e3h) {
   const T3Tri tr = tris[blockIdx.x];
@@ -252,6 +281,7 @@ __global__ void __launch_bounds__(T3_THREADS, 3) k_t3_energy(const T3Tri* __rest
   __shared__ int64_t syo[EXP_MAX_G];  // Y^T block of pair irrep hh: element offset (rows bc, columns a)
   __shared__ int32_t sna[EXP_MAX_G];  // its columns
   __shared__ double red[2][T3_THREADS / 32];
+  __shared__ float2 sev[DS ? T3_SEV : 1];  // DS: energies of the irrep of a, split (its first T3_SEV)
   const int P[3] = {tr.i, tr.j, tr.k};
   const int gijk = (T.go[tr.i] + T.go[tr.j] + T.go[tr.k]) % G;
   if (int(threadIdx.x) < G) {
@@ -259,12 +289,14 @@ __global__ void __launch_bounds__(T3_THREADS, 3) k_t3_energy(const T3Tri* __rest
     syo[hh] = yoff[int64_t(blockIdx.x) * G + hh];
     sna[hh] = T.vcnt[((gijk - hh) % G + G) % G];
   }
-  __syncthreads();
   const int ga = ((gijk - h) % G + G) % G;
   const int na = T.vcnt[ga], a0 = T.voff[ga];
   const int n = T.npair[h];
   const int32_t* pr = T.pairs + T.poff[h];
   const double* ev = eps + o;
+  if (DS)
+    for (int x = threadIdx.x; x < min(na, T3_SEV); x += blockDim.x) sev[x] = ds_split(ev[a0 + x]);
+  __syncthreads();
   const double eijk = eps[tr.i] + eps[tr.j] + eps[tr.k];
   const int gx[3] = {T.go[tr.i], T.go[tr.j], T.go[tr.k]};
   const int Yx[3] = {tr.j, tr.i, tr.j}, Zx[3] = {tr.k, tr.k, tr.i};
@@ -284,12 +316,12 @@ __global__ void __launch_bounds__(T3_THREADS, 3) k_t3_energy(const T3Tri* __rest
     double pr_re = 0.0, pr_im = 0.0;                          // FP64 path: this pair's sum
     float2 ar = make_float2(0.f, 0.f), ai = make_float2(0.f, 0.f);  // DS path
     const float2 dbc_ds = DS ? ds_split(dbc) : make_float2(0.f, 0.f);
+    const int hac = (ga + gc) % G, hab = (ga + gb) % G;
     for (int a = a0; a < a0 + na && a < b; ++a) {
       // c_abc = Y(a; bc) - Y(b; ac) + Y(c; ab)
-      const int hac = (ga + gc) % G, hab = (ga + gb) % G;
       const int cac = T.pidx[a * v + c] - 1, cab = T.pidx[a * v + b] - 1;
-      const cplx y1 = Y(a, h, u), y2 = Y(b, hac, cac), y3 = Y(c, hab, cab);
-      if (DS) {
+      const T3Elem<DS> y1 = Y(a, h, u), y2 = Y(b, hac, cac), y3 = Y(c, hab, cab);
+      if constexpr (DS) {
         const dsc cc = dsc_add(dsc_sub(dsc_of(y1), dsc_of(y2)), dsc_of(y3));
         // d_abc = P(i/jk) P(a/bc) t_i^a <bc||jk>: only t1 of matching irreps is nonzero
         dsc d = dsc{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
@@ -302,7 +334,7 @@ __global__ void __launch_bounds__(T3_THREADS, 3) k_t3_energy(const T3Tri* __rest
           if (gc == gx[w]) { const dsc s = dsc_mul(dsc_of(t1[int64_t(x) * v + c]), dsc_of(Vv(b, a, y, z))); d = neg ? dsc_add(d, s) : dsc_sub(d, s); }
         }
         const dsc wv = dsc_add(cc, d);
-        const float2 rD = ds_rcp(ds_add(dbc_ds, ds_neg(ds_split(ev[a]))));
+        const float2 rD = ds_rcp(ds_add(dbc_ds, ds_neg(a - a0 < T3_SEV ? sev[a - a0] : ds_split(ev[a]))));
         // conj(w) c / D
         const float2 pre = ds_add(ds_mul(wv.re, cc.re), ds_mul(wv.im, cc.im));
         const float2 pim = ds_add(ds_mul(wv.re, cc.im), ds_neg(ds_mul(wv.im, cc.re)));
@@ -702,6 +734,13 @@ void ccsd_t(Ctx& c, int inst, int block, exp_t3_info* info, double* per_triple) 
     sc.A = emu_set_new(c, c.cfg.n_slices, false);
     sc.B = emu_set_new(c, c.cfg.n_slices, true);
     emu_set_slice(c, sc.A, bmats, Bbuf);
+    // t1 and <bc||jk> serve the energy kernel alone from here on
+    const int64_t n1 = int64_t(o) * v, nV = int64_t(o) * o * v * v;
+    for (const auto& x : {std::make_pair(t1d, n1), std::make_pair(Vd, nV)}) {
+      k_t3_ds<<<unsigned(std::max<int64_t>(1, std::min<int64_t>((x.second + T3_THREADS - 1) / T3_THREADS, 4096))), T3_THREADS,
+                0, c.stream>>>(x.first, x.second);
+      KCHECK(c);
+    }
   }
 
   // block size: the largest whose segment and Y^T buffers fit the budget
@@ -799,7 +838,7 @@ void ccsd_t(Ctx& c, int inst, int block, exp_t3_info* info, double* per_triple) 
         mark();
         // Y^T = sum of the segment products, for every (triple, h) of the batch
         if (emulated) {
-          emu_set_multiply(c, sc.A, sc.B, bp.prods, Yt, make_double2(1.0, 0.0));
+          emu_set_multiply(c, sc.A, sc.B, bp.prods, Yt, 0, true);
         } else {
           for (int w = 0; w < 3; ++w) {
             std::vector<GemmProb>& fp = bp.fprods[w];
@@ -826,7 +865,8 @@ void ccsd_t(Ctx& c, int inst, int block, exp_t3_info* info, double* per_triple) 
         mark();
         const dim3 eg(unsigned(bp.tris.size()), unsigned(G));
         if (emulated)
-          k_t3_energy<true><<<eg, T3_THREADS, 0, c.stream>>>(d_tris, DT.T, Yt, d_yoff, t1d, Vd, eps, o, v, e3h);
+          k_t3_energy<true><<<eg, T3_THREADS, 0, c.stream>>>(
+              d_tris, DT.T, (const float4*)Yt, d_yoff, (const float4*)t1d, (const float4*)Vd, eps, o, v, e3h);
         else
           k_t3_energy<false><<<eg, T3_THREADS, 0, c.stream>>>(d_tris, DT.T, Yt, d_yoff, t1d, Vd, eps, o, v, e3h);
         KCHECK(c);
