@@ -9,6 +9,9 @@
 #include "engine.h"
 #include "fpbits.h"
 
+// terms to a leaf, leaves to a branch of a thread's sum
+constexpr int GEMM_LEAF = 32, GEMM_FAN = 16;
+
 // One output element per thread (lanes = 1), or per group of `lanes` threads that
 // share its K (lanes a power of two, then a fixed butterfly; above a warp a fixed
 // sum over the group's warps in shared memory).
@@ -21,12 +24,21 @@
 // partitions of all SMs get the same share.  So: outputs numbered along the rows of
 // all blocks (no padded rows or columns at any shape), CTAs of two warps (the last
 // wave is then a small part of the launch), and K shared among lanes only where the
-// outputs alone do not fill the chip.  Measured against 64 x 64 shared-memory tiles
+// outputs alone do not fill the chip.
+//
+// The K terms of a thread are summed in leaves of LEAF, FAN leaves to a branch, the
+// branches in sequence, so that the rounding error grows with LEAF + FAN + K / (LEAF
+// FAN) rather than with K, for two FP64 additions in 4 LEAF FMAs.  rms error of an
+// output (in 2^-53, normal terms) in one sequence per thread -> so: 300 x 300 x 4000
+// 2374 -> 258, 700 x 700 x 8000 4487 -> 390, 109 x 109 x 12000 (8 lanes) 2454 -> 444 (in
+// ranges of 256 terms: 605, 1456, 1087); 1024^3 6.92 -> 7.04 ms.
+//
+// Measured against 64 x 64 shared-memory tiles
 // (with a warp per output for small products), TFLOP/s of complex work, exp_zgemm:
 // 1024^3 1.17 -> 1.22, 300^3 0.16 -> 0.81, 6000 x 24 x 400 0.27 -> 0.98, 64 x 64 x 5000
 // 0.14 -> 0.70; one CCSD iteration at o=10 v=40 8.2 -> 2.1 ms, at o=40 v=200 Z8 278 ->
 // 203 ms (1.22 TFLOP/s), (T) at o=24 v=120 Z8 1940 -> 97 ms.
-template <int THREADS>
+template <int THREADS, int LEAF, int FAN>
 __global__ void __launch_bounds__(THREADS) k_gemm_fp64(const GemmProb* __restrict__ probs, int n_probs,
                                                        const cplx* __restrict__ A, const cplx* __restrict__ B,
                                                        cplx* __restrict__ C, int64_t ais, int64_t bis, int64_t cis,
@@ -48,14 +60,35 @@ __global__ void __launch_bounds__(THREADS) k_gemm_fp64(const GemmProb* __restric
     const cplx* a = A + blockIdx.y * ais + P.a + m * P.K + lane;
     const cplx* b = B + blockIdx.y * bis + P.b + int64_t(lane) * P.N + n;
     const int64_t bstep = int64_t(lanes) * P.N;
-#pragma unroll 4
-    for (int k = lane; k < P.K; k += lanes, a += lanes, b += bstep) {
+    double lr = 0.0, li = 0.0;
+    auto term = [&] {
       const cplx x = *a, y = *b;
-      sr = fma(x.x, y.x, sr);
-      sr = fma(-x.y, y.y, sr);
-      si = fma(x.x, y.y, si);
-      si = fma(x.y, y.x, si);
+      lr = fma(x.x, y.x, lr);
+      lr = fma(-x.y, y.y, lr);
+      li = fma(x.x, y.y, li);
+      li = fma(x.y, y.x, li);
+      a += lanes;
+      b += bstep;
+    };
+    // (the same number of whole leaves for all lanes: one that has a term more would
+    // send the warp through both loops)
+    const int full = P.K / (lanes * LEAF);
+    for (int f = 0; f < full;) {
+      double br = 0.0, bi = 0.0;  // a branch
+      for (const int end = min(f + FAN, full); f < end; ++f) {
+#pragma unroll 8
+        for (int q = 0; q < LEAF; ++q) term();
+        br += lr;
+        bi += li;
+        lr = li = 0.0;
+      }
+      sr += br;
+      si += bi;
     }
+#pragma unroll 4
+    for (int k = full * LEAF * lanes + lane; k < P.K; k += lanes) term();
+    sr += lr;
+    si += li;
   }
   for (int o = min(lanes, 32) >> 1; o; o >>= 1) {
     sr += __shfl_xor_sync(0xffffffffu, sr, o);
@@ -100,10 +133,10 @@ void launch_gemm_fp64(Ctx& c, const GemmPlan& g, const cplx* A, const cplx* B, c
   if (blocks > INT32_MAX) throw ExpError{EXP_EINVAL, "FP64 product: too many outputs in one launch"};
   const dim3 grid(unsigned(blocks), c.ninst);
   if (threads == 64)
-    k_gemm_fp64<64><<<grid, 64, 0, c.stream>>>(g.d_probs, g.n_probs, A, B, C, ais, bis, cis, alpha, beta, g.n_out, g.lanes);
+    k_gemm_fp64<64, GEMM_LEAF, GEMM_FAN><<<grid, 64, 0, c.stream>>>(g.d_probs, g.n_probs, A, B, C, ais, bis, cis, alpha, beta, g.n_out, g.lanes);
   else
-    k_gemm_fp64<GEMM_MAX_LANES><<<grid, GEMM_MAX_LANES, 0, c.stream>>>(g.d_probs, g.n_probs, A, B, C, ais, bis, cis, alpha,
-                                                                      beta, g.n_out, g.lanes);
+    k_gemm_fp64<GEMM_MAX_LANES, GEMM_LEAF, GEMM_FAN><<<grid, GEMM_MAX_LANES, 0, c.stream>>>(
+        g.d_probs, g.n_probs, A, B, C, ais, bis, cis, alpha, beta, g.n_out, g.lanes);
   KCHECK(c);
 }
 
