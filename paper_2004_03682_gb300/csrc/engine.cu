@@ -545,9 +545,9 @@ GemmPlan make_gemm_plan(Ctx& c, const Layout& A, const Layout& B, const Layout& 
     g.flops_mac += M * N * K;
     g.h_probs.push_back(p);
   }
-  g.lanes = gemm_lanes(c, g.n_out * c.ninst, maxK);
   g.matvec = maxN <= 2 || (g.flops_mac * c.ninst < (int64_t(1) << 22) &&
                            (maxK >= 32 || g.n_out * c.ninst <= (int64_t(1) << 18)));
+  gemm_lanes(c, g, maxK);
   g.n_probs = int(g.h_probs.size());
   if (g.n_probs) {
     g.d_probs = (GemmProb*)c.dalloc(g.h_probs.size() * sizeof(GemmProb));

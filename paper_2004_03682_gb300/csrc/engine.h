@@ -152,6 +152,7 @@ struct GemmPlan {
   int n_probs = 0;
   int64_t n_out = 0;      // output elements per instance
   int lanes = 1;          // threads per output of the FP64 product (gemm_lanes)
+  int leaf = 0;           // its sums pairwise in leaves of this many terms (0: not pairwise)
   int64_t flops_mac = 0;  // complex MACs per instance
   bool matvec = false;    // matrix-vector or small: stays FP64 where a short K would go to k_gemm_ds
   std::vector<GemmProb> h_probs;
@@ -201,7 +202,7 @@ void launch_tau3(Ctx& c, cplx* tau, cplx* taut, cplx* zeta, int64_t dst_is, cons
                  int n_chunks);
 void launch_gemm_fp64(Ctx& c, const GemmPlan& g, const cplx* A, const cplx* B, cplx* C,
                       int64_t a_is, int64_t b_is, int64_t c_is, cplx alpha, bool beta);
-int gemm_lanes(const Ctx& c, int64_t outputs, int kmax);
+void gemm_lanes(const Ctx& c, GemmPlan& g, int kmax);
 // double-single SIMT product for short contractions (every K <= 16) under the
 // emulated precision: ds_wanted decides, ds_prepare builds its tile list once
 bool ds_wanted(Ctx& c, const GemmPlan& g);

@@ -11,6 +11,28 @@
 
 // terms to a leaf, leaves to a branch of a thread's sum
 constexpr int GEMM_LEAF = 32, GEMM_FAN = 16;
+constexpr int GEMM_PAIRWISE_K = 512;  // longest K, and terms a thread, of pairwise sums
+constexpr int GEMM_PAIRWISE_TERMS = 64;
+
+// sum of the next N terms (a power of two), leaves of LEAF terms added pairwise
+template <int N, int LEAF>
+__device__ __forceinline__ cplx pairwise(const cplx*& a, const cplx*& b, int64_t astep, int64_t bstep) {
+  if constexpr (N <= LEAF) {
+    double r = 0.0, i = 0.0;
+#pragma unroll
+    for (int q = 0; q < N; ++q, a += astep, b += bstep) {
+      const cplx x = *a, y = *b;
+      r = fma(x.x, y.x, r);
+      r = fma(-x.y, y.y, r);
+      i = fma(x.x, y.y, i);
+      i = fma(x.y, y.x, i);
+    }
+    return make_double2(r, i);
+  } else {
+    const cplx u = pairwise<N / 2, LEAF>(a, b, astep, bstep), v = pairwise<N / 2, LEAF>(a, b, astep, bstep);
+    return make_double2(u.x + v.x, u.y + v.y);
+  }
+}
 
 // One output element per thread (lanes = 1), or per group of `lanes` threads that
 // share its K (lanes a power of two, then a fixed butterfly; above a warp a fixed
@@ -26,9 +48,9 @@ constexpr int GEMM_LEAF = 32, GEMM_FAN = 16;
 // wave is then a small part of the launch), and K shared among lanes only where the
 // outputs alone do not fill the chip.
 //
-// The K terms of a thread are summed in leaves of LEAF, FAN leaves to a branch, the
-// branches in sequence, so that the rounding error grows with LEAF + FAN + K / (LEAF
-// FAN) rather than with K, for two FP64 additions in 4 LEAF FMAs.  rms error of an
+// The K terms of a thread are summed in leaves of 32, 16 leaves to a branch, the
+// branches in sequence, so that the rounding error grows with 32 + 16 + K / 512
+// rather than with K, for two FP64 additions in 128 FMAs.  rms error of an
 // output (in 2^-53, normal terms) in one sequence per thread -> so: 300 x 300 x 4000
 // 2374 -> 258, 700 x 700 x 8000 4487 -> 390, 109 x 109 x 12000 (8 lanes) 2454 -> 444 (in
 // ranges of 256 terms: 605, 1456, 1087); 1024^3 6.92 -> 7.04 ms.
@@ -38,7 +60,7 @@ constexpr int GEMM_LEAF = 32, GEMM_FAN = 16;
 // 1024^3 1.17 -> 1.22, 300^3 0.16 -> 0.81, 6000 x 24 x 400 0.27 -> 0.98, 64 x 64 x 5000
 // 0.14 -> 0.70; one CCSD iteration at o=10 v=40 8.2 -> 2.1 ms, at o=40 v=200 Z8 278 ->
 // 203 ms (1.22 TFLOP/s), (T) at o=24 v=120 Z8 1940 -> 97 ms.
-template <int THREADS, int LEAF, int FAN>
+template <int THREADS, int LEAF>
 __global__ void __launch_bounds__(THREADS) k_gemm_fp64(const GemmProb* __restrict__ probs, int n_probs,
                                                        const cplx* __restrict__ A, const cplx* __restrict__ B,
                                                        cplx* __restrict__ C, int64_t ais, int64_t bis, int64_t cis,
@@ -60,35 +82,48 @@ __global__ void __launch_bounds__(THREADS) k_gemm_fp64(const GemmProb* __restric
     const cplx* a = A + blockIdx.y * ais + P.a + m * P.K + lane;
     const cplx* b = B + blockIdx.y * bis + P.b + int64_t(lane) * P.N + n;
     const int64_t bstep = int64_t(lanes) * P.N;
-    double lr = 0.0, li = 0.0;
-    auto term = [&] {
-      const cplx x = *a, y = *b;
-      lr = fma(x.x, y.x, lr);
-      lr = fma(-x.y, y.y, lr);
-      li = fma(x.x, y.y, li);
-      li = fma(x.y, y.x, li);
-      a += lanes;
-      b += bstep;
-    };
-    // (the same number of whole leaves for all lanes: one that has a term more would
-    // send the warp through both loops)
-    const int full = P.K / (lanes * LEAF);
-    for (int f = 0; f < full;) {
-      double br = 0.0, bi = 0.0;  // a branch
-      for (const int end = min(f + FAN, full); f < end; ++f) {
+    if constexpr (LEAF > 0) {  // pairwise
+      int left = P.K > lane ? (P.K - lane - 1) / lanes + 1 : 0;
+      auto add = [&](cplx t) {
+        sr += t.x;
+        si += t.y;
+      };
+      for (; left >= 16; left -= 16) add(pairwise<16, LEAF>(a, b, lanes, bstep));
+      if (left & 8) add(pairwise<8, LEAF>(a, b, lanes, bstep));
+      if (left & 4) add(pairwise<4, LEAF>(a, b, lanes, bstep));
+      if (left & 2) add(pairwise<2, LEAF>(a, b, lanes, bstep));
+      if (left & 1) add(pairwise<1, LEAF>(a, b, lanes, bstep));
+    } else {
+      double lr = 0.0, li = 0.0;
+      auto term = [&] {
+        const cplx x = *a, y = *b;
+        lr = fma(x.x, y.x, lr);
+        lr = fma(-x.y, y.y, lr);
+        li = fma(x.x, y.y, li);
+        li = fma(x.y, y.x, li);
+        a += lanes;
+        b += bstep;
+      };
+      // (the same number of whole leaves for all lanes: one that has a term more would
+      // send the warp through both loops)
+      const int full = P.K / (lanes * GEMM_LEAF);
+      for (int f = 0; f < full;) {
+        double br = 0.0, bi = 0.0;  // a branch
+        for (const int end = min(f + GEMM_FAN, full); f < end; ++f) {
 #pragma unroll 8
-        for (int q = 0; q < LEAF; ++q) term();
-        br += lr;
-        bi += li;
-        lr = li = 0.0;
+          for (int q = 0; q < GEMM_LEAF; ++q) term();
+          br += lr;
+          bi += li;
+          lr = li = 0.0;
+        }
+        sr += br;
+        si += bi;
       }
-      sr += br;
-      si += bi;
-    }
 #pragma unroll 4
-    for (int k = full * LEAF * lanes + lane; k < P.K; k += lanes) term();
-    sr += lr;
-    si += li;
+      for (int k = full * GEMM_LEAF * lanes + lane; k < P.K; k += lanes) term();
+      sr += lr;
+      si += li;
+    }
   }
   for (int o = min(lanes, 32) >> 1; o; o >>= 1) {
     sr += __shfl_xor_sync(0xffffffffu, sr, o);
@@ -117,11 +152,28 @@ __global__ void __launch_bounds__(THREADS) k_gemm_fp64(const GemmProb* __restric
 // four warps, else the smallest power of two that does, while each lane keeps at
 // least four k (a shorter share costs more butterfly additions than it saves: each
 // halving of a lane's k adds two additions to four FMAs a k).
-int gemm_lanes(const Ctx& c, int64_t outputs, int kmax) {
-  const int64_t want = int64_t(std::max(c.sm_count, 1)) * 4 * 4 * 32;
-  int lanes = 1;
-  while (lanes < GEMM_MAX_LANES && outputs * lanes < want && kmax >= 8 * lanes) lanes *= 2;
-  return lanes;
+//
+// Matrix-vector products and small ones (GemmPlan::matvec) keep the accuracy of the
+// kernel they ran on before, a warp per output with a term or a few per lane: one
+// sequence per thread had up to five times its error.  K above GEMM_PAIRWISE_K is shared
+// by a warp at least (a lane's sequence is then as short as there); below, a thread adds
+// its terms pairwise, in leaves of two (K < 128, where the pairs decide) or four.  rms
+// error of an output in 2^-53 and time, a warp per output / one sequence per thread /
+// now: 360 x 360 x 32 9.0, 157 us / 20.3, 32 us / 9.1, 42 us; 100 x 100 x 400 53, 42 us
+// / 89, 35 us / 44, 40 us; 100000 x 1 x 5000 549, 3395 us / 3035, 3988 us / 265, 3413
+// us.  The lanes also read a row of A side by side: with one thread to a row, the last
+// product was slower than a warp per output.
+void gemm_lanes(const Ctx& c, GemmPlan& g, int kmax) {
+  const int64_t want = int64_t(std::max(c.sm_count, 1)) * 4 * 4 * 32, outputs = g.n_out * c.ninst;
+  g.lanes = 1;
+  while (g.lanes < GEMM_MAX_LANES && outputs * g.lanes < want && kmax >= 8 * g.lanes) g.lanes *= 2;
+  if (!g.matvec) return;
+  if (kmax > GEMM_PAIRWISE_K) {
+    g.lanes = std::max(g.lanes, 32);
+  } else if (g.lanes <= 32) {
+    while (kmax > GEMM_PAIRWISE_TERMS * g.lanes) g.lanes *= 2;
+    g.leaf = kmax < 128 ? 2 : 4;
+  }
 }
 
 void launch_gemm_fp64(Ctx& c, const GemmPlan& g, const cplx* A, const cplx* B, cplx* C, int64_t ais,
@@ -131,12 +183,12 @@ void launch_gemm_fp64(Ctx& c, const GemmPlan& g, const cplx* A, const cplx* B, c
   const int64_t per = threads / g.lanes;
   const int64_t blocks = (g.n_out + per - 1) / per;
   if (blocks > INT32_MAX) throw ExpError{EXP_EINVAL, "FP64 product: too many outputs in one launch"};
-  const dim3 grid(unsigned(blocks), c.ninst);
-  if (threads == 64)
-    k_gemm_fp64<64, GEMM_LEAF, GEMM_FAN><<<grid, 64, 0, c.stream>>>(g.d_probs, g.n_probs, A, B, C, ais, bis, cis, alpha, beta, g.n_out, g.lanes);
-  else
-    k_gemm_fp64<GEMM_MAX_LANES, GEMM_LEAF, GEMM_FAN><<<grid, GEMM_MAX_LANES, 0, c.stream>>>(
-        g.d_probs, g.n_probs, A, B, C, ais, bis, cis, alpha, beta, g.n_out, g.lanes);
+  const auto kernel = threads > 64 ? k_gemm_fp64<GEMM_MAX_LANES, 0>
+                      : g.leaf == 2 ? k_gemm_fp64<64, 2>
+                      : g.leaf == 4 ? k_gemm_fp64<64, 4>
+                                    : k_gemm_fp64<64, 0>;
+  kernel<<<dim3(unsigned(blocks), c.ninst), threads, 0, c.stream>>>(g.d_probs, g.n_probs, A, B, C, ais, bis, cis, alpha,
+                                                                    beta, g.n_out, g.lanes);
   KCHECK(c);
 }
 

@@ -40,3 +40,14 @@ def _ranges(K, r=256):
 @pytest.mark.parametrize("M,N,K", [(300, 300, 4000), (400, 400, 5000), (109, 109, 12000), (700, 130, 8000), (64, 64, 100000)])
 def test_long_sums_are_as_accurate_as_ranges_of_256_terms(M, N, K):
     assert _rms_error(M, N, K) < _ranges(K)
+
+
+# one warp to an output: a sequence per lane, then the lanes pairwise
+def _warp(K):
+    return U * np.sqrt(32 * _sequence(K / 32 if K > 32 else 1) * min(K, 32) / 32 + 4.0 / 12.0 * 2 * K * np.ceil(np.log2(min(K, 32))))
+
+
+@pytest.mark.parametrize("M,N,K", [(20000, 1, 5000), (20000, 2, 2000), (1, 3000, 1000), (100000, 1, 40), (60000, 2, 16),
+                                   (360, 360, 32), (290, 290, 48), (200, 200, 100), (100, 100, 400), (64, 64, 1000)])
+def test_small_and_matrix_vector_products_are_as_accurate_as_a_warp_per_output(M, N, K):
+    assert _rms_error(M, N, K) < _warp(K)
