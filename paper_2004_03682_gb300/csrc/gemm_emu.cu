@@ -30,6 +30,7 @@
 #include <cstdio>
 #include <mutex>
 #include <string>
+#include <type_traits>
 
 #include "emu.h"
 #include "fpbits.h"
@@ -48,11 +49,48 @@ constexpr int EMU_GM = 8;      // default row tiles per group of the GEMM work o
 #define ALPHA_POS_BIAS 64
 #define ALPHA_NEG_BIAS 64
 
-// Real output columns per tile: as many as fit 256 TMEM columns.  Wider tiles copy fewer
-// bytes and issue fewer MMAs per output (an MMA of N columns takes N / 2 clocks, but about
-// 45 at least).  4096^3, 64 columns against 48: three slices 3.83 -> 2.96 ms, four 4.37 ->
+// Real output columns per tile.  Wider tiles copy fewer bytes and issue fewer MMAs per
+// output (an MMA of N columns takes N / 2 clocks, but about 45 at least); S diagonals of
+// BN columns fill at most 256 TMEM columns, and a warp of the epilogue takes a multiple of
+// 8 of them.  4096^3, 64 columns against 48: three slices 3.83 -> 2.96 ms, four 4.37 ->
 // 3.48 ms.
 constexpr int bn_of(int S) { return S <= 4 ? 64 : S == 5 ? 48 : 32; }
+constexpr int BN_NARROW = 48;  // the other width of three and four slices
+
+// Width of the tiles of a product or operand set with these output columns: a tile of 64
+// columns costs more than one of 48 (N = 24: 4000 rows, K = 200 13.1 against 16.6 us at
+// three slices, 14.3 against 18.1 at four; 20000 rows, K = 1000 61.8 against 64.4 and 74.5
+// against 77.2), so it has to save tiles.  33 of 32: the long-K ratio.
+template <typename Cols>
+int tile_columns(int S, int nh, int n, Cols cols) {
+  if (S > 4) return bn_of(S);
+  int64_t wide = 0, narrow = 0;
+  for (int k = 0; k < n; ++k) {
+    const int64_t real = int64_t(nh) * cols(k);  // a complex column is two real ones
+    wide += (real + bn_of(S) - 1) / bn_of(S);
+    narrow += (real + BN_NARROW - 1) / BN_NARROW;
+  }
+  return 32 * narrow <= 33 * wide ? BN_NARROW : bn_of(S);
+}
+
+// f(S, BN) with both as compile-time constants
+template <typename F>
+void by_shape(int S, int bn, F f) {
+  auto narrow = std::integral_constant<int, BN_NARROW>();
+  auto go = [&](auto s) {
+    constexpr int wide = bn_of(decltype(s)::value);
+    if constexpr (wide > BN_NARROW) {
+      if (bn == BN_NARROW) return f(s, narrow);
+    }
+    f(s, std::integral_constant<int, wide>());
+  };
+  switch (S) {
+    case 3: go(std::integral_constant<int, 3>()); break;
+    case 4: go(std::integral_constant<int, 4>()); break;
+    case 5: go(std::integral_constant<int, 5>()); break;
+    default: go(std::integral_constant<int, 6>()); break;
+  }
+}
 
 template <int S, int COLS = bn_of(S)>
 struct Shape {
@@ -950,6 +988,7 @@ static int alpha_code(cplx a) {
 
 struct EmuPlan {
   int S = 5;
+  int bn = 0;  // real columns per tile
   std::vector<EmuProb> h;
   EmuProb* d = nullptr;
   int n_tiles = 0;                    // GEMM work items
@@ -1052,11 +1091,11 @@ bool emu_wanted(Ctx& c, const GemmPlan& g, const std::string&) {
   return g.flops_mac * c.ninst >= int64_t(1) << 22;
 }
 
-template <int S>
+template <int S, int BN>
 static void set_smem_attr() {
   static bool done = false;
   if (!done) {
-    CK(cudaFuncSetAttribute(k_emu_gemm<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, Shape<S>::SMEM));
+    CK(cudaFuncSetAttribute(k_emu_gemm<S, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, Shape<S, BN>::SMEM));
     done = true;
   }
 }
@@ -1085,11 +1124,11 @@ EmuPlan* emu_plan(Ctx& c, const GemmPlan& g, const Tensor* A, const Tensor* B, b
   p->a_const = a_const;
   p->b_const = b_const;
   p->d_err = st->d_err;
-  const int BN = bn_of(p->S);
+  const int nh = c.cfg.real_arith ? 1 : 2;  // real operands: no Im half, one B row per column
+  const int BN = p->bn = tile_columns(p->S, nh, int(g.h_probs.size()), [&](int k) { return g.h_probs[k].N; });
   int64_t asl = 0, bsl = 0, aex = 0, bex = 0;
   int64_t au0 = 0, bu0 = 0;
   int64_t tiles_mn = 0;
-  const int nh = c.cfg.real_arith ? 1 : 2;  // real operands: no Im half, one B row per column
   const int ocols = nh == 2 ? BN / 2 : BN;
   for (auto& q : g.h_probs)
     tiles_mn += int64_t((q.M + BM - 1) / BM) * ((q.N + ocols - 1) / ocols);
@@ -1234,12 +1273,12 @@ extern "C" exp_status exp_test_emu_wait(int skip_kblock, double wait_ms) {
 }
 
 // The GEMM launch of a plan (plus its split-K reduction) into C.
-template <int S>
+template <int S, int BN>
 static void launch_product(Ctx& c, EmuPlan* p, cplx* C, int64_t cis, cplx alpha, bool beta, bool reduce) {
   const int np = int(p->h.size());
-  set_smem_attr<S>();
+  set_smem_attr<S, BN>();
   const int n_work = p->n_tiles * c.ninst;
-  k_emu_gemm<S><<<dim3(std::min(n_work, std::max(c.sm_count, 1))), Shape<S>::THREADS, Shape<S>::SMEM,
+  k_emu_gemm<S, BN><<<dim3(std::min(n_work, std::max(c.sm_count, 1))), Shape<S, BN>::THREADS, Shape<S, BN>::SMEM,
                   c.stream>>>(
       p->d, np, p->n_tiles, n_work, p->gm, p->asl, p->bsl, p->aex, p->bex, C, p->asl_is, p->bsl_is, p->aex_is,
       p->bex_is, cis, alpha, p->red_elems ? ALPHA_GENERAL : alpha_code(alpha), beta ? 1 : 0, p->d_err, p->d_ws, p->ws_is,
@@ -1260,7 +1299,7 @@ static void launch_product(Ctx& c, EmuPlan* p, cplx* C, int64_t cis, cplx alpha,
 // group -- and keep the fastest.  Trial launches write a scratch output; split-K
 // partials are exact, so no candidate changes the result.  Skipped while the
 // stream is being captured and for one-off products.
-template <int S>
+template <int S, int BN>
 static void autotune(Ctx& c, EmuPlan* p, int64_t cis, cplx alpha) {
   p->tuned = true;
   if (!c.autotune) return;
@@ -1291,10 +1330,10 @@ static void autotune(Ctx& c, EmuPlan* p, int64_t cis, cplx alpha) {
     upload(c, p->d, p->h.data(), sizeof(EmuProb) * p->h.size());
     for (int g : gms) {
       p->gm = g;
-      if (!warm) launch_product<S>(c, p, st->tune_buf, cis, alpha, false, true);  // one warm-up
+      if (!warm) launch_product<S, BN>(c, p, st->tune_buf, cis, alpha, false, true);  // one warm-up
       warm = true;
       CK(cudaEventRecord(e0, c.stream));
-      launch_product<S>(c, p, st->tune_buf, cis, alpha, false, true);
+      launch_product<S, BN>(c, p, st->tune_buf, cis, alpha, false, true);
       CK(cudaEventRecord(e1, c.stream));
       CK(cudaEventSynchronize(e1));
       float ms = 0.f;
@@ -1313,14 +1352,14 @@ static void autotune(Ctx& c, EmuPlan* p, int64_t cis, cplx alpha) {
             best_m, best_gm, best_ms);
 }
 
-template <int S>
+template <int S, int BN>
 static void run_s(Ctx& c, EmuPlan* p, const cplx* A, const cplx* B, cplx* C, int64_t ais, int64_t bis, int64_t cis,
                   cplx alpha, bool beta, bool gemm_only) {
   const int np = int(p->h.size());
   if (p->asl_arena) p->asl = (__nv_bfloat16*)c.slice_arena.base;
   if (p->bsl_arena) p->bsl = (__nv_bfloat16*)c.slice_arena.base + p->bsl_off;
   if (gemm_only) {  // the tensor-core product alone, on the slices already in place
-    launch_product<S>(c, p, C, cis, alpha, beta, false);
+    launch_product<S, BN>(c, p, C, cis, alpha, beta, false);
     return;
   }
   EmuStageTimer tm(c.profile, c.stream);
@@ -1352,14 +1391,14 @@ static void run_s(Ctx& c, EmuPlan* p, const cplx* A, const cplx* B, cplx* C, int
     k_col_exp<<<dim3(p->n_colexp, c.ninst), 256, 0, c.stream>>>(p->d, np, B, bis, p->bex, p->bex_is);
     KCHECK(c);
     tm.mark(3);
-    k_split_b<S><<<dim3(split_blocks(p->n_bunits, c.sm_count), c.ninst), 256, 0, c.stream>>>(
+    k_split_b<S, BN><<<dim3(split_blocks(p->n_bunits, c.sm_count), c.ninst), 256, 0, c.stream>>>(
         p->d, np, p->n_bunits, B, bis, p->bex, p->bex_is, p->bsl, p->bsl_is);
     KCHECK(c);
     if (p->b_const) p->b_ready = true;
   }
   tm.mark(4);
-  if (!p->tuned) autotune<S>(c, p, cis, alpha);
-  launch_product<S>(c, p, C, cis, alpha, beta, false);
+  if (!p->tuned) autotune<S, BN>(c, p, cis, alpha);
+  launch_product<S, BN>(c, p, C, cis, alpha, beta, false);
   tm.mark(5);
   if (p->red_elems) {
     int mks = 1;
@@ -1375,12 +1414,7 @@ static void run_s(Ctx& c, EmuPlan* p, const cplx* A, const cplx* B, cplx* C, int
 void emu_run(Ctx& c, EmuPlan* p, const GemmPlan&, const cplx* A, const cplx* B, cplx* C, int64_t ais, int64_t bis,
              int64_t cis, cplx alpha, bool beta, bool gemm_only) {
   if (p->n_tiles == 0) return;
-  switch (p->S) {
-    case 3: run_s<3>(c, p, A, B, C, ais, bis, cis, alpha, beta, gemm_only); break;
-    case 4: run_s<4>(c, p, A, B, C, ais, bis, cis, alpha, beta, gemm_only); break;
-    case 5: run_s<5>(c, p, A, B, C, ais, bis, cis, alpha, beta, gemm_only); break;
-    default: run_s<6>(c, p, A, B, C, ais, bis, cis, alpha, beta, gemm_only); break;
-  }
+  by_shape(p->S, p->bn, [&](auto s, auto n) { run_s<s(), n()>(c, p, A, B, C, ais, bis, cis, alpha, beta, gemm_only); });
 }
 
 void emu_release(Ctx& c) {
@@ -1399,6 +1433,7 @@ void emu_release(Ctx& c) {
 // A-side fields of one member and the B-side fields of another.
 struct EmuSet {
   int S = 5;
+  int bn = 0;  // B side: real columns per tile
   bool b_side = false;
   int nh = 2;
   std::vector<EmuProb> h;  // one record per member, the fields of its side filled
@@ -1454,7 +1489,7 @@ static void grow(Ctx& c, T*& p, int64_t& cap, int64_t need) {
   p = (T*)c.dalloc(sizeof(T) * size_t(cap));
 }
 
-template <int S>
+template <int S, int BN>
 static void set_slice_s(Ctx& c, EmuSet* s, const cplx* src) {
   const int np = int(s->h.size());
   k_fill_int<<<dim3(int(std::max<int64_t>(1, std::min<int64_t>((s->n_ex + 255) / 256, 1024)))), 256, 0, c.stream>>>(
@@ -1473,14 +1508,14 @@ static void set_slice_s(Ctx& c, EmuSet* s, const cplx* src) {
     k_split_a<S, false><<<dim3(split_blocks(s->units, c.sm_count), 1), 256, 0, c.stream>>>(s->d, np, s->units, src, 0,
                                                                                           s->ex, 0, s->sl, 0);
   else
-    k_split_b<S><<<dim3(split_blocks(s->units, c.sm_count), 1), 256, 0, c.stream>>>(s->d, np, s->units, src, 0, s->ex,
+    k_split_b<S, BN><<<dim3(split_blocks(s->units, c.sm_count), 1), 256, 0, c.stream>>>(s->d, np, s->units, src, 0, s->ex,
                                                                                    0, s->sl, 0);
   KCHECK(c);
 }
 
 void emu_set_slice(Ctx& c, EmuSet* s, const std::vector<EmuSetMat>& mats, const cplx* src) {
   const int S = s->S, nh = s->nh;
-  const int BN = bn_of(S);
+  const int BN = s->bn = s->b_side ? tile_columns(S, nh, int(mats.size()), [&](int k) { return mats[k].rows; }) : bn_of(S);
   const int ocols = nh == 2 ? BN / 2 : BN;
   s->h.clear();
   int64_t sl = 0, ex = 0, u0 = 0, scan = 0;
@@ -1543,19 +1578,14 @@ void emu_set_slice(Ctx& c, EmuSet* s, const std::vector<EmuSetMat>& mats, const 
   grow(c, s->ex, s->ex_cap, s->n_ex);
   grow(c, s->d, s->d_cap, int64_t(s->h.size()));
   upload_async(c, s->d, s->h.data(), sizeof(EmuProb) * s->h.size());
-  switch (S) {
-    case 3: set_slice_s<3>(c, s, src); break;
-    case 4: set_slice_s<4>(c, s, src); break;
-    case 5: set_slice_s<5>(c, s, src); break;
-    default: set_slice_s<6>(c, s, src); break;
-  }
+  by_shape(S, s->bn, [&](auto sl, auto n) { set_slice_s<sl(), n()>(c, s, src); });
 }
 
-template <int S>
+template <int S, int BN>
 static void set_multiply_s(Ctx& c, const EmuProb* d, int np, int n_tiles, const EmuSet* A, const EmuSet* B, cplx* C,
                            int alpha_k, bool ds_out, int* gerr, const int* t2p) {
-  set_smem_attr<S>();
-  k_emu_gemm<S><<<dim3(std::min(n_tiles, std::max(c.sm_count, 1))), Shape<S>::THREADS, Shape<S>::SMEM,
+  set_smem_attr<S, BN>();
+  k_emu_gemm<S, BN><<<dim3(std::min(n_tiles, std::max(c.sm_count, 1))), Shape<S, BN>::THREADS, Shape<S, BN>::SMEM,
                   c.stream>>>(
       d, np, n_tiles, n_tiles, EMU_GM, A->sl, B->sl, A->ex, B->ex, C, 0, 0, 0, 0, 0, make_double2(1.0, 0.0),
       alpha_k + ALPHA_POS_BIAS, 0, gerr, nullptr, 0, emu_wait_test(), t2p, ds_out ? 1 : 0);
@@ -1653,12 +1683,7 @@ void emu_set_multiply(Ctx& c, const EmuSet* A, const EmuSet* B, const std::vecto
     KCHECK(c);
     t2p = st->set_t2p;
   }
-  switch (S) {
-    case 3: set_multiply_s<3>(c, st->set_d, np, nt, A, B, C, alpha_k, ds_out, st->d_err, t2p); break;
-    case 4: set_multiply_s<4>(c, st->set_d, np, nt, A, B, C, alpha_k, ds_out, st->d_err, t2p); break;
-    case 5: set_multiply_s<5>(c, st->set_d, np, nt, A, B, C, alpha_k, ds_out, st->d_err, t2p); break;
-    default: set_multiply_s<6>(c, st->set_d, np, nt, A, B, C, alpha_k, ds_out, st->d_err, t2p); break;
-  }
+  by_shape(S, B->bn, [&](auto s, auto n) { set_multiply_s<s(), n()>(c, st->set_d, np, nt, A, B, C, alpha_k, ds_out, st->d_err, t2p); });
 }
 
 // ---------------------------------------------------------------------------
@@ -1722,7 +1747,7 @@ exp_status noalloc_launch(cudaStream_t st, unsigned char* base, int M, int N, in
                           cplx* Cout, cplx alpha, int beta, int sms, std::string& err) {
   // three and four slices keep tiles of 48 columns here: wider ones would change which
   // problems fit the fixed scratch
-  constexpr int BN = std::min(bn_of(S), 48);
+  constexpr int BN = std::min(bn_of(S), BN_NARROW);
   using SH = Shape<S, BN>;
   EmuProb e{};
   e.M = M;
