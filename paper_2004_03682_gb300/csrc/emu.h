@@ -23,16 +23,16 @@ void emu_release(Ctx& c);
 // Operand sets for grouped products whose operand pairing is chosen at run time (the
 // products of the (T) correction).  The members of a set are sliced together; a
 // product pairs an A member (rows x K, row-major) with a B member (K x cols,
-// row-major) of the same K and writes C (rows x cols, row-major) = 2^alpha_k A B, or the
-// sum of up to three such pairs (segments) with equal rows and cols: C = 2^alpha_k
+// row-major) of the same K and writes C (rows x cols, row-major) = A B, or the
+// sum of up to three such pairs (segments) with equal rows and cols: C =
 // sum_w A_w B_w, accumulated exactly over the concatenated K (a product whose
 // segments all have K = 0 leaves its C as it is).  Members of one
 // exponent group (same rows / cols) share their row (A) or column (B) exponents, the
 // maximum over the group; the segments of one product must come from one A group and
 // one B group.  The products of one call share one launch; each product needs a total
 // K short enough for one exact int64 accumulation (K' up to 2^(13 - 7 (S - 6)) KC
-// terms: far above (T)'s).  ds_out: C in double-single, four floats (re.h, re.l, im.h, im.l)
-// an element, |alpha_k| <= 60.
+// terms: far above (T)'s).  C is double-single, four floats (re.h, re.l, im.h, im.l) an
+// element.
 struct EmuSet;
 struct EmuSetMat {
   int64_t src;  // element offset of the member in the source array
@@ -49,6 +49,5 @@ EmuSet* emu_set_new(Ctx& c, int S, bool b_side);
 // lay out the members (growing the set's device buffers when needed), then scan
 // their exponents and write their slice tiles from src
 void emu_set_slice(Ctx& c, EmuSet* s, const std::vector<EmuSetMat>& mats, const cplx* src);
-void emu_set_multiply(Ctx& c, const EmuSet* A, const EmuSet* B, const std::vector<EmuSetProd>& prods, cplx* C,
-                      int alpha_k, bool ds_out);
+void emu_set_multiply(Ctx& c, const EmuSet* A, const EmuSet* B, const std::vector<EmuSetProd>& prods, float4* C);
 void emu_set_free(Ctx& c, EmuSet* s);

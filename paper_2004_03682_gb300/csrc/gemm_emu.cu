@@ -321,14 +321,18 @@ __device__ __forceinline__ EmuWork emu_work(const EmuProb* probs, int nprobs, in
 // The stage ring and the two TMEM accumulator buffers run on across items, so
 // the epilogue of one tile overlaps the MMAs of the next and the producer
 // prefetches across tile boundaries.
-template <int S, int COLS = bn_of(S)>
+// DS: C in double-single and alpha = 1 (operand sets).  A kernel of its own: as a branch of
+// one kernel the conversions lengthened the code of every product's epilogue, which a
+// launch of few tiles runs through once (five slices, 4000 x 24 x 40 12.8 against 10.6 us,
+// 600 x 600 x 100 14.7 against 13.1; three and four alike, six by 0.3 us).
+template <int S, int COLS = bn_of(S), bool DS = false>
 __global__ void __launch_bounds__(Shape<S, COLS>::THREADS, 1)
     k_emu_gemm(const EmuProb* probs, int nprobs, int n_tiles, int n_work, int gm,
                const __nv_bfloat16* __restrict__ Asl, const __nv_bfloat16* __restrict__ Bsl,
                const int* __restrict__ Aex, const int* __restrict__ Bex, cplx* __restrict__ C, int64_t asl_is,
                int64_t bsl_is, int64_t aex_is, int64_t bex_is, int64_t c_is, cplx alpha, int alpha_e, int beta,
                int* __restrict__ gerr, cplx* __restrict__ ws, int64_t ws_is, EmuWaitTest wt,
-               const int* __restrict__ t2p, int ds_out) {
+               const int* __restrict__ t2p) {
   using SH = Shape<S, COLS>;
   constexpr int STAGES = SH::STAGES;
   const unsigned long long wns = wt.wait_ns;
@@ -495,8 +499,9 @@ __global__ void __launch_bounds__(Shape<S, COLS>::THREADS, 1)
       // first output column of this warp
       const int j0 = cpx ? W.nt * (SH::BN / 2) + h * (HW / 2) : W.nt * SH::BN + h * HW;
       const int ei = gi < P.M ? Aex[W.inst * aex_is + P.a_ex + gi] : 0;
-      // the exponent of output column j0 + lane, handed out by shuffle (with 16 epilogue warps
-      // of 16 columns a register per column would spill)
+      // the exponent of output column j0 + lane, handed out by shuffle: a register per column
+      // would add to the spills of 16 epilogue warps of 16 columns (64-column tiles: 96
+      // registers a thread, 16 bytes spilled)
       const int fjl = (lane < (cpx ? HW / 2 : HW) && j0 + lane < P.N) ? Bex[W.inst * bex_is + P.b_ex + j0 + lane] : 0;
       for (int ch = 0; ch < nchunks; ++ch, ++gc) {
         const int buf = gc & 1;
@@ -548,8 +553,8 @@ __global__ void __launch_bounds__(Shape<S, COLS>::THREADS, 1)
             const int gj = j0 + u;
             const int e = ei + __shfl_sync(0xffffffffu, fjl, u) - BETA * (S + 1);
             if (live && gj < P.N) {
-              if (ds_out) {
-                const float2 x = ds_of_i64(alpha_e < 0 ? -R[u] : R[u], e + alpha_k);
+              if constexpr (DS) {
+                const float2 x = ds_of_i64(R[u], e);
                 reinterpret_cast<float4*>(Crow)[gj] = make_float4(x.x, x.y, 0.f, 0.f);
                 continue;
               }
@@ -584,9 +589,8 @@ __global__ void __launch_bounds__(Shape<S, COLS>::THREADS, 1)
           const int gj = j0 + jj;
           const int e = ei + __shfl_sync(0xffffffffu, fjl, jj) - BETA * (S + 1);
           if (live && gj < P.N) {
-            if (ds_out) {
-              const float2 x = ds_of_i64(alpha_e < 0 ? -R[2 * jj] : R[2 * jj], e + alpha_k);
-              const float2 y = ds_of_i64(alpha_e < 0 ? -R[2 * jj + 1] : R[2 * jj + 1], e + alpha_k);
+            if constexpr (DS) {
+              const float2 x = ds_of_i64(R[2 * jj], e), y = ds_of_i64(R[2 * jj + 1], e);
               reinterpret_cast<float4*>(Crow)[gj] = make_float4(x.x, x.y, y.x, y.y);
               continue;
             }
@@ -1091,11 +1095,11 @@ bool emu_wanted(Ctx& c, const GemmPlan& g, const std::string&) {
   return g.flops_mac * c.ninst >= int64_t(1) << 22;
 }
 
-template <int S, int BN>
+template <int S, int BN, bool DS>
 static void set_smem_attr() {
   static bool done = false;
   if (!done) {
-    CK(cudaFuncSetAttribute(k_emu_gemm<S, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, Shape<S, BN>::SMEM));
+    CK(cudaFuncSetAttribute(k_emu_gemm<S, BN, DS>, cudaFuncAttributeMaxDynamicSharedMemorySize, Shape<S, BN>::SMEM));
     done = true;
   }
 }
@@ -1276,13 +1280,13 @@ extern "C" exp_status exp_test_emu_wait(int skip_kblock, double wait_ms) {
 template <int S, int BN>
 static void launch_product(Ctx& c, EmuPlan* p, cplx* C, int64_t cis, cplx alpha, bool beta, bool reduce) {
   const int np = int(p->h.size());
-  set_smem_attr<S, BN>();
+  set_smem_attr<S, BN, false>();
   const int n_work = p->n_tiles * c.ninst;
   k_emu_gemm<S, BN><<<dim3(std::min(n_work, std::max(c.sm_count, 1))), Shape<S, BN>::THREADS, Shape<S, BN>::SMEM,
                   c.stream>>>(
       p->d, np, p->n_tiles, n_work, p->gm, p->asl, p->bsl, p->aex, p->bex, C, p->asl_is, p->bsl_is, p->aex_is,
       p->bex_is, cis, alpha, p->red_elems ? ALPHA_GENERAL : alpha_code(alpha), beta ? 1 : 0, p->d_err, p->d_ws, p->ws_is,
-      emu_wait_test(), nullptr, 0);
+      emu_wait_test(), nullptr);
   KCHECK(c);
   if (reduce && p->red_elems) {
     int mks = 1;
@@ -1583,17 +1587,16 @@ void emu_set_slice(Ctx& c, EmuSet* s, const std::vector<EmuSetMat>& mats, const 
 
 template <int S, int BN>
 static void set_multiply_s(Ctx& c, const EmuProb* d, int np, int n_tiles, const EmuSet* A, const EmuSet* B, cplx* C,
-                           int alpha_k, bool ds_out, int* gerr, const int* t2p) {
-  set_smem_attr<S, BN>();
-  k_emu_gemm<S, BN><<<dim3(std::min(n_tiles, std::max(c.sm_count, 1))), Shape<S, BN>::THREADS, Shape<S, BN>::SMEM,
-                  c.stream>>>(
+                           int* gerr, const int* t2p) {
+  set_smem_attr<S, BN, true>();
+  k_emu_gemm<S, BN, true><<<dim3(std::min(n_tiles, std::max(c.sm_count, 1))), Shape<S, BN>::THREADS, Shape<S, BN>::SMEM,
+                            c.stream>>>(
       d, np, n_tiles, n_tiles, EMU_GM, A->sl, B->sl, A->ex, B->ex, C, 0, 0, 0, 0, 0, make_double2(1.0, 0.0),
-      alpha_k + ALPHA_POS_BIAS, 0, gerr, nullptr, 0, emu_wait_test(), t2p, ds_out ? 1 : 0);
+      ALPHA_POS_BIAS, 0, gerr, nullptr, 0, emu_wait_test(), t2p);
   KCHECK(c);
 }
 
-void emu_set_multiply(Ctx& c, const EmuSet* A, const EmuSet* B, const std::vector<EmuSetProd>& prods, cplx* C,
-                      int alpha_k, bool ds_out) {
+void emu_set_multiply(Ctx& c, const EmuSet* A, const EmuSet* B, const std::vector<EmuSetProd>& prods, float4* C) {
   if (A->b_side || !B->b_side || A->S != B->S || A->nh != B->nh)
     throw ExpError{EXP_EINVAL, "emulated product: operand sets do not match"};
   const int S = A->S;
@@ -1683,7 +1686,9 @@ void emu_set_multiply(Ctx& c, const EmuSet* A, const EmuSet* B, const std::vecto
     KCHECK(c);
     t2p = st->set_t2p;
   }
-  by_shape(S, B->bn, [&](auto s, auto n) { set_multiply_s<s(), n()>(c, st->set_d, np, nt, A, B, C, alpha_k, ds_out, st->d_err, t2p); });
+  by_shape(S, B->bn, [&](auto s, auto n) {
+    set_multiply_s<s(), n()>(c, st->set_d, np, nt, A, B, reinterpret_cast<cplx*>(C), st->d_err, t2p);
+  });
 }
 
 // ---------------------------------------------------------------------------
@@ -1834,7 +1839,7 @@ exp_status noalloc_launch(cudaStream_t st, unsigned char* base, int M, int N, in
   const int n_work = int(tiles_mn * e.ksplit);
   k_emu_gemm<S, BN><<<dim3(unsigned(std::min(n_work, sms)), 1), SH::THREADS, SH::SMEM, st>>>(
       d_probs, 1, n_work, n_work, EMU_GM, asl, bsl, aex, bex, Cout, 0, 0, 0, 0, 0, alpha,
-      e.ksplit > 1 ? ALPHA_GENERAL : alpha_code(alpha), beta, d_err, ws, 0, EmuWaitTest{2000000000ull, -1, 0}, nullptr, 0);
+      e.ksplit > 1 ? ALPHA_GENERAL : alpha_code(alpha), beta, d_err, ws, 0, EmuWaitTest{2000000000ull, -1, 0}, nullptr);
   if (!launched("k_emu_gemm")) return EXP_ECUDA;
   if (e.ksplit > 1) {
     launch_emu_reduce(d_probs, 1, e.ksplit, ws, 0, Cout, 0, aex, 0, bex, 0, S, alpha, beta, int64_t(M) * N, 1, sms, st);

@@ -838,7 +838,7 @@ void ccsd_t(Ctx& c, int inst, int block, exp_t3_info* info, double* per_triple) 
         mark();
         // Y^T = sum of the segment products, for every (triple, h) of the batch
         if (emulated) {
-          emu_set_multiply(c, sc.A, sc.B, bp.prods, Yt, 0, true);
+          emu_set_multiply(c, sc.A, sc.B, bp.prods, (float4*)Yt);
         } else {
           for (int w = 0; w < 3; ++w) {
             std::vector<GemmProb>& fp = bp.fprods[w];

@@ -35,7 +35,7 @@ def test_tile_width(S, M, N, K, cols):
             for s in ((M, K), (K, N)))
     out, names = _kernels(lambda: expgb.zgemm(A, B, precision=expgb.EXP_EMU_BF16, n_slices=S))
     np.testing.assert_array_equal(out.cpu().numpy(), A.cpu().numpy() @ B.cpu().numpy())
-    assert f"k_emu_gemm<{S}, {cols}" in names
+    assert f"k_emu_gemm<{S}, {cols}, false>" in names  # and without the code of the double-single outputs
 
 
 # each slice fewer costs 7 bits: 1e-9 at six slices
@@ -52,4 +52,4 @@ def test_triples_on_either_width(S, rel, no, nv, G, cols):
     orc = triples.per_triple(t1, t2, ccsd.Blocks(integrals.integrals(prob), integrals.fock(prob), no))
     ref = np.array([orc[i, j, k] for k in range(no) for j in range(k) for i in range(j)])
     assert np.abs(e3 - ref).max() < rel * np.abs(ref).max()
-    assert f"k_emu_gemm<{S}, {cols}" in names
+    assert f"k_emu_gemm<{S}, {cols}, true>" in names
