@@ -57,21 +57,36 @@ constexpr int EMU_GM = 8;      // default row tiles per group of the GEMM work o
 constexpr int bn_of(int S) { return S <= 4 ? 64 : S == 5 ? 48 : 32; }
 constexpr int BN_NARROW = 48;  // the other width of three and four slices
 
-// Width of the tiles of a product or operand set with these output columns: a tile of 64
-// columns costs more than one of 48 (N = 24: 4000 rows, K = 200 13.1 against 16.6 us at
-// three slices, 14.3 against 18.1 at four; 20000 rows, K = 1000 61.8 against 64.4 and 74.5
-// against 77.2), so it has to save tiles.  33 of 32: the long-K ratio.
-template <typename Cols>
-int tile_columns(int S, int nh, int n, Cols cols) {
-  if (S > 4) return bn_of(S);
+// Relative time of one tile of `cols` columns and nkb k-blocks at three and four slices: an
+// epilogue by its columns, k-blocks nearly by their copies of A (2000 x 2000, four slices, a
+// wave of tiles of 48 / 64 columns: K = 20 5.4 / 7.1 us, K = 250 10.4 / 12.5, K = 2048 62 / 66).
+static double tile_cost(int cols, int nkb) { return cols == BN_NARROW ? 1.0 + 0.08 * nkb : 1.36 + 0.083 * nkb; }
+
+struct TileCount {  // output tiles of a product at both widths, and their time
   int64_t wide = 0, narrow = 0;
-  for (int k = 0; k < n; ++k) {
-    const int64_t real = int64_t(nh) * cols(k);  // a complex column is two real ones
-    wide += (real + bn_of(S) - 1) / bn_of(S);
-    narrow += (real + BN_NARROW - 1) / BN_NARROW;
+  double wide_cost = 0.0, narrow_cost = 0.0;
+  // tm row tiles; cols real output columns
+  void add(int S, int64_t tm, int64_t cols, int nkb) {
+    const int64_t w = tm * ((cols + bn_of(S) - 1) / bn_of(S)), n = tm * ((cols + BN_NARROW - 1) / BN_NARROW);
+    wide += w;
+    narrow += n;
+    wide_cost += double(w) * tile_cost(bn_of(S), nkb);
+    narrow_cost += double(n) * tile_cost(BN_NARROW, nkb);
   }
-  return 32 * narrow <= 33 * wide ? BN_NARROW : bn_of(S);
-}
+  // The width: 64 columns have to save tiles, and where K is too short to be split, waves of
+  // tiles.  48 / 64 columns at four slices: 4000 x 24 x 200 (32 tiles or 32) 14.4 / 18.2 us,
+  // 20000 x 24 x 1000 71.6 / 76.6, 600 x 600 x 100 (125 or 95, one wave) 12.0 / 13.9,
+  // 4000 x 150 x 20 (224 or 160, two waves) 14.0 / 15.0; 12000 x 100 x 300 (470 or 376)
+  // 49.3 / 44.8.
+  int columns(int S, int64_t sms, bool splits) const {
+    if (S > 4) return bn_of(S);
+    auto time = [&](int64_t tiles, double cost) {
+      if (tiles == 0 || (splits && tiles < 2 * sms)) return cost;
+      return cost * double((tiles + sms - 1) / sms * sms) / double(tiles);
+    };
+    return time(narrow, narrow_cost) <= time(wide, wide_cost) ? BN_NARROW : bn_of(S);
+  }
+};
 
 // f(S, BN) with both as compile-time constants
 template <typename F>
@@ -1068,9 +1083,9 @@ static void layout_work(EmuPlan* p, int64_t sms, double mult) {
 struct BKey {
   const void* ptr;
   int64_t is;
-  int S;
+  int S, bn;
   std::vector<int64_t> probs;  // (b_src, K, N) per problem
-  bool operator==(const BKey& o) const { return ptr == o.ptr && is == o.is && S == o.S && probs == o.probs; }
+  bool operator==(const BKey& o) const { return ptr == o.ptr && is == o.is && S == o.S && bn == o.bn && probs == o.probs; }
 };
 
 struct EmuState {
@@ -1129,7 +1144,15 @@ EmuPlan* emu_plan(Ctx& c, const GemmPlan& g, const Tensor* A, const Tensor* B, b
   p->b_const = b_const;
   p->d_err = st->d_err;
   const int nh = c.cfg.real_arith ? 1 : 2;  // real operands: no Im half, one B row per column
-  const int BN = p->bn = tile_columns(p->S, nh, int(g.h_probs.size()), [&](int k) { return g.h_probs[k].N; });
+  const int64_t sms = std::max(c.sm_count, 1);
+  TileCount tc;
+  bool long_k = false;
+  for (auto& q : g.h_probs) {
+    const int nkb = kp_of(q.K, nh) / KB;
+    tc.add(p->S, int64_t((q.M + BM - 1) / BM) * c.ninst, int64_t(nh) * q.N, nkb);
+    long_k |= nkb >= 2 * KC_BLOCKS;
+  }
+  const int BN = p->bn = tc.columns(p->S, sms, long_k);
   int64_t asl = 0, bsl = 0, aex = 0, bex = 0;
   int64_t au0 = 0, bu0 = 0;
   int64_t tiles_mn = 0;
@@ -1137,7 +1160,6 @@ EmuPlan* emu_plan(Ctx& c, const GemmPlan& g, const Tensor* A, const Tensor* B, b
   for (auto& q : g.h_probs)
     tiles_mn += int64_t((q.M + BM - 1) / BM) * ((q.N + ocols - 1) / ocols);
   tiles_mn *= c.ninst;
-  const int64_t sms = std::max(c.sm_count, 1);
   p->fuse_a = true;
   for (auto& q : g.h_probs) {
     EmuProb e{};
@@ -1200,7 +1222,7 @@ EmuPlan* emu_plan(Ctx& c, const GemmPlan& g, const Tensor* A, const Tensor* B, b
   p->aex = (int*)c.dalloc(sizeof(int) * p->aex_is * c.ninst);
   // B slices: reuse those of an earlier plan that reads the same tensor the same way
   // (plans run in creation order every iteration, so the owner has sliced it already)
-  BKey key{B ? (const void*)B->d : nullptr, B ? B->is : 0, p->S, {}};
+  BKey key{B ? (const void*)B->d : nullptr, B ? B->is : 0, p->S, p->bn, {}};
   for (auto& e : p->h) { key.probs.push_back(e.b_src); key.probs.push_back(e.K); key.probs.push_back(e.N); }
   if (B && b_shareable)
     for (auto& kv : st->bowners)
@@ -1519,7 +1541,10 @@ static void set_slice_s(Ctx& c, EmuSet* s, const cplx* src) {
 
 void emu_set_slice(Ctx& c, EmuSet* s, const std::vector<EmuSetMat>& mats, const cplx* src) {
   const int S = s->S, nh = s->nh;
-  const int BN = s->bn = s->b_side ? tile_columns(S, nh, int(mats.size()), [&](int k) { return mats[k].rows; }) : bn_of(S);
+  // (products of up to three members, many at a time: no last wave to speak of)
+  TileCount tc;
+  for (const EmuSetMat& m : mats) tc.add(S, 1, int64_t(nh) * m.rows, 3 * (kp_of(m.K, nh) / KB));
+  const int BN = s->bn = tc.columns(S, 1, true);
   const int ocols = nh == 2 ? BN / 2 : BN;
   s->h.clear();
   int64_t sl = 0, ex = 0, u0 = 0, scan = 0;

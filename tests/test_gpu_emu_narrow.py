@@ -1,5 +1,6 @@
 """GPU: the width of the emulated product's tiles at three and four slices: 48 real columns where 64 would not
-save a tile, bit-exact either way; and (T), whose operand sets are laid out in those tiles, on both."""
+save a tile, or a wave of them at short K, bit-exact either way; and (T), whose operand sets are laid out in
+those tiles, on both."""
 import numpy as np
 import pytest
 
@@ -26,9 +27,10 @@ def _kernels(f):
 
 
 @pytest.mark.parametrize("S", [3, 4])
-@pytest.mark.parametrize("M,N,K,cols", [(300, 1, 70, 48), (300, 24, 70, 48), (300, 25, 70, 64), (140, 32, 600, 64),
-                                        (140, 33, 600, 48), (140, 48, 40, 48), (140, 49, 40, 64), (150, 72, 300, 48),
-                                        (150, 73, 300, 64), (200, 700, 100, 64)])
+@pytest.mark.parametrize("M,N,K,cols", [(300, 1, 70, 48), (300, 24, 70, 48), (300, 25, 70, 48), (140, 32, 600, 64),
+                                        (140, 33, 600, 48), (140, 48, 40, 48), (140, 49, 40, 48), (150, 72, 300, 48),
+                                        (150, 73, 1100, 64), (600, 600, 100, 48), (4000, 150, 20, 48),
+                                        (20000, 25, 100, 64), (12000, 100, 300, 64)])
 def test_tile_width(S, M, N, K, cols):
     rng = np.random.default_rng(S + M + 10 * N + 100 * K)
     A, B = (torch.tensor(rng.integers(-8, 9, s) + 1j * rng.integers(-8, 9, s), dtype=torch.complex128, device="cuda")
