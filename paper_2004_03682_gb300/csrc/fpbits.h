@@ -74,15 +74,15 @@ __device__ __forceinline__ float2 ds_of_i64(long long R, int e) {
   hm += rem + (hm & 1u) > (1ull << 39) ? 1u : 0u;
   const long long r = (long long)(m - ((unsigned long long)hm << 40));  // the rest, |r| <= 2^39
   const int fe = 190 + e - lz;  // biased exponent of hm 2^(40 + e - lz), hm in [2^23, 2^24]
-  // beyond the range of FP32: infinite, as the conversion gives
-  const int fc = fe < 255 ? fe : 255;
-  // a significand rounded up to 2^24 carries into the exponent field
-  const float h = __uint_as_float(sgn | ((unsigned(fc) << 23) + (fc == 255 ? 0u : hm - 0x800000u)));
+  // a significand rounded up to 2^24 carries into the exponent field; beyond the range of
+  // FP32, by the exponent or that carry: infinite without a rest, as ds_split gives
+  const unsigned hb = fe < 255 ? (unsigned(fe) << 23) + (hm - 0x800000u) : 0x7F800000u;
+  const float h = __uint_as_float(sgn | hb);
   const unsigned lb = __float_as_uint(__int2float_rn(int(r >> 9)));  // l = this 2^(9 + e - lz)
   const int le = int((lb >> 23) & 0xFF) + 9 + e - lz;
   const float l = __uint_as_float(((lb & 0x807FFFFFu) | (unsigned(le) << 23)) ^ sgn);
   const bool tiny = fe < 1 || R == 0;
-  return make_float2(tiny ? 0.f : h, tiny || fc == 255 || le < 1 || (r < 512 && r >= 0) ? 0.f : l);
+  return make_float2(tiny ? 0.f : h, tiny || hb == 0x7F800000u || le < 1 || (r < 512 && r >= 0) ? 0.f : l);
 }
 
 // signed integer significand and exponent of a float: f = m 2^e
