@@ -73,3 +73,26 @@ def test_bf16_guess_by_element_count(o, v, g):
     _, _, y = _forward(p, np.stack([np.abs(t) / 0.05, -D / 10.0, va / va.max()], -1).reshape(-1, 3))
     want = (1 + y[:, 0] + 1j * y[:, 1]).reshape(t.shape) * t
     assert np.abs(got - want).max() < TOL * np.abs(want).max()
+
+
+def test_bf16_guess_of_many_instances_by_element():
+    """More elements to an instance than one sweep of its CTAs takes, a ragged end, a trained output layer: every
+    instance against the oracle."""
+    n, o, v = 64, 6, 23  # 19044 elements an instance; 8 waves of 3 CTAs on each SM are 57 CTAs of 128 an instance
+    probs = [syn.make_problem(40 + k, o, v, 1) for k in range(n)]
+    ctx = expgb.from_problems(probs)
+    ctx.init_integrals([p.seed for p in probs], scale_mult=[0.5 + k / n for k in range(n)])
+    expgb.Mlp(seed=5).apply(ctx)  # untrained: the first-order amplitudes
+    first = [ctx.get_amplitudes(k)[1].cpu().numpy() for k in range(n)]
+    m, p = expgb.Mlp(seed=1, bf16=True), _params(4)
+    m.params(set=p)
+    m.apply(ctx)
+    for k, (prob, t) in enumerate(zip(probs, first)):
+        got = ctx.get_amplitudes(k)[1].cpu().numpy()
+        D = (prob.eps_occ[:, None, None, None] + prob.eps_occ[:, None, None] - prob.eps_virt[:, None] - prob.eps_virt)
+        va = np.abs(t) * np.abs(D)
+        _, _, y = _forward(p, np.stack([np.abs(t) / 0.05, -D / 10.0, va / va.max()], -1).reshape(-1, 3))
+        want = (1 + y[:, 0] + 1j * y[:, 1]).reshape(t.shape) * t
+        assert np.abs(want - t).max() > 0.05 * np.abs(t).max()  # the output layer counts
+        assert np.abs(got - want).max() < TOL * np.abs(want).max()
+    ctx.close()
