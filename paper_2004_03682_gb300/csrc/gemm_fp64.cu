@@ -9,8 +9,7 @@
 #include "engine.h"
 #include "fpbits.h"
 
-// terms to a leaf, leaves to a branch of a thread's sum
-constexpr int GEMM_LEAF = 32, GEMM_FAN = 16;
+constexpr int GEMM_LEAF = 64;  // terms to a leaf of a thread's sum
 constexpr int GEMM_PAIRWISE_K = 512;  // longest K, and terms a thread, of pairwise sums
 constexpr int GEMM_PAIRWISE_TERMS = 64;
 
@@ -48,12 +47,14 @@ __device__ __forceinline__ cplx pairwise(const cplx*& a, const cplx*& b, int64_t
 // wave is then a small part of the launch), and K shared among lanes only where the
 // outputs alone do not fill the chip.
 //
-// The K terms of a thread are summed in leaves of 32, 16 leaves to a branch, the
-// branches in sequence, so that the rounding error grows with 32 + 16 + K / 512
-// rather than with K, for two FP64 additions in 128 FMAs.  rms error of an
-// output (in 2^-53, normal terms) in one sequence per thread -> so: 300 x 300 x 4000
-// 2374 -> 258, 700 x 700 x 8000 4487 -> 390, 109 x 109 x 12000 (8 lanes) 2454 -> 444 (in
-// ranges of 256 terms: 605, 1456, 1087); 1024^3 6.92 -> 7.04 ms.
+// The K terms of a thread are summed in leaves of 64, the leaves in sequence, so that
+// the rounding error grows with 64 + K / 64 rather than with K, for two FP64 additions
+// in 256 FMAs.  rms error of an output (in 2^-53, normal terms) in one sequence per
+// thread -> so: 300 x 300 x 4000 2374 -> 377, 700 x 700 x 8000 4487 -> 563, 109 x 109 x
+// 12000 (8 lanes) 2454 -> 595 (in ranges of 256 terms: 605, 1456, 1087); 1024^3 6.91 ->
+// 6.98 ms.  Leaves of 32 in branches of 16 have two thirds of that error and take 7.05 ms.
+// (Loads of 8 terms ahead serve the few CTAs of 256 threads, 16 x 16 x 500000 1.30 -> 1.01
+// ms; where CTAs fill the chip 4 are better, 400 x 400 x 5000 5.74 -> 5.53 ms.)
 //
 // Measured against 64 x 64 shared-memory tiles
 // (with a warp per output for small products), TFLOP/s of complex work, exp_zgemm:
@@ -107,17 +108,12 @@ __global__ void __launch_bounds__(THREADS) k_gemm_fp64(const GemmProb* __restric
       // (the same number of whole leaves for all lanes: one that has a term more would
       // send the warp through both loops)
       const int full = P.K / (lanes * GEMM_LEAF);
-      for (int f = 0; f < full;) {
-        double br = 0.0, bi = 0.0;  // a branch
-        for (const int end = min(f + GEMM_FAN, full); f < end; ++f) {
-#pragma unroll 8
-          for (int q = 0; q < GEMM_LEAF; ++q) term();
-          br += lr;
-          bi += li;
-          lr = li = 0.0;
-        }
-        sr += br;
-        si += bi;
+      for (int f = 0; f < full; ++f) {
+#pragma unroll(THREADS > 64 ? 8 : 4)
+        for (int q = 0; q < GEMM_LEAF; ++q) term();
+        sr += lr;
+        si += li;
+        lr = li = 0.0;
       }
 #pragma unroll 4
       for (int k = full * GEMM_LEAF * lanes + lane; k < P.K; k += lanes) term();
@@ -160,7 +156,7 @@ __global__ void __launch_bounds__(THREADS) k_gemm_fp64(const GemmProb* __restric
 // its terms pairwise, in leaves of two (K < 128, where the pairs decide) or four.  rms
 // error of an output in 2^-53 and time, a warp per output / one sequence per thread /
 // now: 360 x 360 x 32 9.0, 157 us / 20.3, 32 us / 9.1, 42 us; 100 x 100 x 400 53, 42 us
-// / 89, 35 us / 44, 40 us; 100000 x 1 x 5000 549, 3395 us / 3035, 3988 us / 265, 3413
+// / 89, 35 us / 44, 40 us; 100000 x 1 x 5000 549, 3395 us / 3035, 3988 us / 339, 3371
 // us.  The lanes also read a row of A side by side: with one thread to a row, the last
 // product was slower than a warp per output.
 void gemm_lanes(const Ctx& c, GemmPlan& g, int kmax) {
