@@ -154,7 +154,7 @@ struct GemmPlan {
   int lanes = 1;          // threads per output of the FP64 product (gemm_lanes)
   int leaf = 0;           // its sums pairwise in leaves of this many terms (0: not pairwise)
   int64_t flops_mac = 0;  // complex MACs per instance
-  bool matvec = false;    // matrix-vector or small: stays FP64 where a short K would go to k_gemm_ds
+  bool matvec = false;    // matrix-vector or small (make_gemm_plan)
   std::vector<GemmProb> h_probs;
   GemmProb* d_ds = nullptr;  // double-single SIMT tiles (k_gemm_ds), set by ds_prepare
   int ds_tiles = 0;
