@@ -316,7 +316,8 @@ constexpr int LDB = W + 8;       // BF16 row stride in shared memory: 272 B, row
 constexpr int GT = 128;          // samples per group of the gradient: 16 per warp, four tiles of TS
 constexpr int LDG = W + 4;       // FP32 row stride of gz1
 constexpr int BF_THREADS = 256;
-constexpr int BF_APPLY = 128;  // threads of the inference CTA: 3 of them an SM at up to 170 registers
+// threads of the inference CTA: 3 of them an SM at up to 170 registers (168 used, 136 bytes spilled)
+constexpr int BF_APPLY = 128;
 constexpr int BF_PARAMS = W * 16 + W * 8 + W * 4;      // per unit: (W1 row, b1), W3 column, b2
 constexpr int BF_FWD_SMEM = W * LDB * 2 + BF_PARAMS;   // + W2
 constexpr int BF_APPLY_SMEM = BF_FWD_SMEM + BF_APPLY * LDB * 2;  // + h2
@@ -707,6 +708,7 @@ struct exp_mlp {
   exp_allocator alloc{};
   cudaStream_t stream = nullptr;
   int bf = 1;
+  int sms = 1;
   int step = 0;
   float* P = nullptr;
   float* G = nullptr;
@@ -755,6 +757,9 @@ extern "C" exp_status exp_mlp_create(const exp_allocator* alloc, void* stream, u
   m->alloc = *alloc;
   m->stream = (cudaStream_t)stream;
   m->bf = bf16 ? 1 : 0;
+  int dev = 0;
+  CK(cudaGetDevice(&dev));
+  CK(cudaDeviceGetAttribute(&m->sms, cudaDevAttrMultiProcessorCount, dev));
   m->P = (float*)m->al(sizeof(float) * NPARAM);
   m->G = (float*)m->al(sizeof(float) * NPARAM);
   m->M1 = (float*)m->al(sizeof(float) * NPARAM);
@@ -892,7 +897,7 @@ extern "C" exp_status exp_mlp_add_training_data(exp_mlp* m, exp_ctx* x) {
 static void grad_batch(exp_mlp* m, const float* X, const float2* TM, const float2* TG, const int* idx, int64_t b0,
                        int64_t nb) {
   CK(cudaMemsetAsync(m->G, 0, sizeof(float) * NPARAM, m->stream));
-  const int blocks = int(std::min<int64_t>((nb + TS - 1) / TS, 304));
+  const int blocks = int(std::min<int64_t>((nb + TS - 1) / TS, 2 * m->sms));
   if (m->bf) {
     k_mlp_grad_bf<<<blocks, BF_THREADS, BF_GRAD_SMEM, m->stream>>>(m->P, X, TM, TG, idx, int(b0), int(nb), 1.f / float(nb),
                                                                    m->G, m->d_loss);
@@ -999,7 +1004,7 @@ extern "C" exp_status exp_mlp_apply(exp_mlp* m, exp_ctx* x) {
   if (m->bf) {
     // three CTAs an SM are resident; eight waves' worth over all instances, each keeping its
     // parameters for many elements
-    const int64_t most = std::max<int64_t>(1, (8 * 3 * 152 + c.ninst - 1) / c.ninst);
+    const int64_t most = std::max<int64_t>(1, (8 * 3 * m->sms + c.ninst - 1) / c.ninst);
     const int blocks = int(std::max<int64_t>(1, std::min<int64_t>((c.n2 + BF_APPLY - 1) / BF_APPLY, most)));
     k_mlp_apply_bf<<<dim3(blocks, c.ninst), BF_APPLY, BF_APPLY_SMEM, c.stream>>>(m->P, Vd->d, Vd->is, c.d_D, c.d_T, c.namp,
                                                                                  c.n1, c.n2, vm);
