@@ -58,7 +58,11 @@
 namespace {
 
 constexpr int T3_THREADS = 256;
-constexpr int T3_SEV = 512;  // split orbital energies a CTA of the energy kernel keeps
+// Split orbital energies a CTA of the energy kernel keeps; it splits the others at each use.  An
+// irrep of more than 512 virtuals does not fit the device in the emulated precision (its block of
+// the packed <ab||cd> alone takes 276 GB, the slices of that more), so that branch only keeps
+// the kernel right at any size.
+constexpr int T3_SEV = 512;
 
 // ---------------------------------------------------------------------------
 // Index tables of one context (irrep-sorted local indices; global spinor index =
