@@ -316,6 +316,7 @@ constexpr int LDB = W + 8;       // BF16 row stride in shared memory: 272 B, row
 constexpr int GT = 128;          // samples per group of the gradient: 16 per warp, four tiles of TS
 constexpr int LDG = W + 4;       // FP32 row stride of gz1
 constexpr int BF_THREADS = 256;
+constexpr int BF_PART = (NPARAM + 31) / 32 * 32;  // row stride of the CTAs' shares of the gradient
 // threads of the inference CTA: 3 of them an SM at up to 170 registers (168 used, 136 bytes spilled)
 constexpr int BF_APPLY = 128;
 constexpr int BF_PARAMS = W * 16 + W * 8 + W * 4;      // per unit: (W1 row, b1), W3 column, b2
@@ -428,11 +429,13 @@ __device__ __forceinline__ void bf_layer2(const BfParams& p, const uint32_t (&a)
 // group meet in shared memory for the sums over samples: gW2 = gz2^T h1 on the tensor
 // cores (warp w the 16 rows u = 16w.., kept in registers over all tiles), the others in
 // FP32, one chain per thread in sample order (a sum per tile for W1, b1 and b2, one running
-// sum for W3 and b3).  One atomicAdd per entry and CTA at the end.
+// sum for W3 and b3).  Each CTA writes its share; k_mlp_fold adds them in a fixed order, so
+// that equal samples give equal parameters in every run (summed by atomics, the shares'
+// order differed from run to run, and with it the last bits of all that training led to).
 __global__ void __launch_bounds__(BF_THREADS, 1)
     k_mlp_grad_bf(const float* __restrict__ P, const float* __restrict__ X, const float2* __restrict__ TM,
                   const float2* __restrict__ TG, const int* __restrict__ idx, int b0, int nb, float inv_n,
-                  float* __restrict__ grad, double* __restrict__ loss) {
+                  float* __restrict__ part, double* __restrict__ lpart) {
   extern __shared__ __align__(16) uint8_t bsm[];
   const BfParams p = bf_load(P, bsm);
   __syncthreads();
@@ -606,23 +609,54 @@ __global__ void __launch_bounds__(BF_THREADS, 1)
     }
     __syncthreads();
   }
+  float* out = part + int64_t(blockIdx.x) * BF_PART;
 #pragma unroll
   for (int nt = 0; nt < 16; ++nt)
 #pragma unroll
     for (int r = 0; r < 2; ++r)
-      atomicAdd(reinterpret_cast<float2*>(&grad[OFF_W2 + (16 * warp + g + 8 * r) * W + 8 * nt + 2 * t]),
-                make_float2(gW2[nt][2 * r], gW2[nt][2 * r + 1]));
-  atomicAdd(&grad[OFF_W3 + threadIdx.x], cW3);
-  if (cu == 0) atomicAdd(&grad[OFF_B3 + co], cb3);
+      *reinterpret_cast<float2*>(&out[OFF_W2 + (16 * warp + g + 8 * r) * W + 8 * nt + 2 * t]) =
+          make_float2(gW2[nt][2 * r], gW2[nt][2 * r + 1]);
+  out[OFF_W3 + threadIdx.x] = cW3;
+  if (cu == 0) out[OFF_B3 + co] = cb3;
   if (co == 0) {
-    atomicAdd(&grad[OFF_B2 + cu], cb2);
+    out[OFF_B2 + cu] = cb2;
   } else {
-    atomicAdd(&grad[OFF_B1 + cu], cb1);
+    out[OFF_B1 + cu] = cb1;
 #pragma unroll
-    for (int f = 0; f < NF; ++f) atomicAdd(&grad[OFF_W1 + cu * NF + f], cW1[f]);
+    for (int f = 0; f < NF; ++f) out[OFF_W1 + cu * NF + f] = cW1[f];
   }
   for (int o = 16; o; o >>= 1) lacc += __shfl_xor_sync(0xffffffffu, lacc, o);
-  if (lane == 0) atomicAdd(loss, lacc * inv_n);
+  if (lane == 0) lpart[int64_t(blockIdx.x) * (BF_THREADS / 32) + warp] = lacc * inv_n;
+}
+
+// The gradient and the loss from the shares of n CTAs, each entry summed in one order: 32
+// entries a CTA, its warp w the shares w, w + 8, ..., then the warps in turn; the last CTA
+// adds the loss.
+__global__ void __launch_bounds__(BF_THREADS) k_mlp_fold(const float* __restrict__ part, const double* __restrict__ lpart,
+                                                         int n, float* __restrict__ grad, double* __restrict__ loss) {
+  constexpr int NW = BF_THREADS / 32;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (blockIdx.x == gridDim.x - 1) {
+    if (warp) return;
+    double s = 0.0;
+    for (int k = lane; k < n * NW; k += 32) s += lpart[k];
+    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) *loss += s;
+    return;
+  }
+  __shared__ float sums[NW][32];
+  const int k = blockIdx.x * 32 + lane;
+  float s = 0.f;
+  if (k < NPARAM) {
+#pragma unroll 8
+    for (int c = warp; c < n; c += NW) s += part[int64_t(c) * BF_PART + k];
+  }
+  sums[warp][lane] = s;
+  __syncthreads();
+  if (warp || k >= NPARAM) return;
+#pragma unroll
+  for (int w = 1; w < NW; ++w) s += sums[w][lane];
+  grad[k] = s;
 }
 
 // Inference, bf16 mode: 32 elements per warp step, one per lane for the features, layer 3
@@ -715,6 +749,8 @@ struct exp_mlp {
   float* M1 = nullptr;
   float* M2 = nullptr;
   double* d_loss = nullptr;
+  float* part = nullptr;    // bf16 mode: the CTAs' shares of the gradient and the loss
+  double* lpart = nullptr;
   float* X = nullptr;
   float2* TM = nullptr;
   float2* TG = nullptr;
@@ -896,12 +932,18 @@ extern "C" exp_status exp_mlp_add_training_data(exp_mlp* m, exp_ctx* x) {
 
 static void grad_batch(exp_mlp* m, const float* X, const float2* TM, const float2* TG, const int* idx, int64_t b0,
                        int64_t nb) {
-  CK(cudaMemsetAsync(m->G, 0, sizeof(float) * NPARAM, m->stream));
-  const int blocks = int(std::min<int64_t>((nb + TS - 1) / TS, 2 * m->sms));
+  const int most = 2 * m->sms, blocks = int(std::min<int64_t>((nb + TS - 1) / TS, most));
   if (m->bf) {
+    if (!m->lpart) {
+      m->part = (float*)m->al(sizeof(float) * BF_PART * most);
+      m->lpart = (double*)m->al(sizeof(double) * (BF_THREADS / 32) * most);
+    }
     k_mlp_grad_bf<<<blocks, BF_THREADS, BF_GRAD_SMEM, m->stream>>>(m->P, X, TM, TG, idx, int(b0), int(nb), 1.f / float(nb),
-                                                                   m->G, m->d_loss);
+                                                                   m->part, m->lpart);
+    CK(cudaGetLastError());
+    k_mlp_fold<<<BF_PART / 32 + 1, BF_THREADS, 0, m->stream>>>(m->part, m->lpart, blocks, m->G, m->d_loss);
   } else {
+    CK(cudaMemsetAsync(m->G, 0, sizeof(float) * NPARAM, m->stream));
     k_mlp_grad<<<blocks, 256, MLP_SMEM, m->stream>>>(m->P, X, TM, TG, idx, int(b0), int(nb), 1.f / float(nb), m->G,
                                                      m->d_loss);
   }

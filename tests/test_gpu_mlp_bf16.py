@@ -96,3 +96,20 @@ def test_bf16_guess_of_many_instances_by_element():
         assert np.abs(want - t).max() > 0.05 * np.abs(t).max()  # the output layer counts
         assert np.abs(got - want).max() < TOL * np.abs(want).max()
     ctx.close()
+
+
+def test_bf16_training_repeats_bit_for_bit():
+    probs = [syn.make_problem(70 + k, 6, 22, 1) for k in range(8)]
+    ctx = expgb.from_problems(probs, conv_tol=1e-6, max_iter=200)
+    ctx.init_integrals([p.seed for p in probs], scale_mult=[0.4] * len(probs))
+    ctx.iterate(200, raise_numeric=False)
+    runs = []
+    for _ in range(3):
+        m = expgb.Mlp(seed=3, bf16=True)
+        m.add_training_data(ctx)
+        assert m.n_samples > 32 * 304
+        runs.append((m.train(4, batch=16384, lr=2e-3, seed=1), m.params()))
+    ctx.close()
+    for losses, params in runs[1:]:
+        np.testing.assert_array_equal(losses, runs[0][0])
+        np.testing.assert_array_equal(params, runs[0][1])
