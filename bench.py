@@ -67,8 +67,9 @@ DEFAULT_WORKLOAD = "ccsd_z8_o60_v400"
 WORKLOAD = WORKLOADS[DEFAULT_WORKLOAD]
 METRIC = "ccsd_iterations_per_s"
 UNIT = "iter/s"
-FP64_NOMINAL_TFLOPS = 1.25      # GB300 nominal dense FP64
-BF16_NOMINAL_TFLOPS = 2250.0    # GB300 nominal dense BF16
+# FP64 peak: the SMs' FP64 pipe takes two FMAs a clock (k_gemm_fp64 runs at 1.23 TFLOP/s), 152 SMs at 2070 MHz
+FP64_TFLOPS = 4 * 152 * 2.07e9 / 1e12
+FP64_SRC = "FP64 = 2 FMAs per clock and SM, 152 SMs, 2070 MHz"
 
 
 def peaks():
@@ -523,11 +524,11 @@ def run_triples(args):
                     "unit": "TFLOP/s", "frac": ach / pk["bf16"], "traffic": None,
                     "peak_src": f"{pk['src']} bf16 dense (burst)", "ms_per_evaluation": mp}
         else:
-            peak = pk["bf16"] * FP64_NOMINAL_TFLOPS / BF16_NOMINAL_TFLOPS
+            peak = FP64_TFLOPS
             ach = info["macs_run"] * 8 / (mp * 1e-3) / 1e12
             roof = {"bound": "tensor", "kernel": "k_gemm_fp64 ((T) products)", "achieved": ach, "peak": peak,
                     "unit": "TFLOP/s", "frac": ach / peak, "traffic": None,
-                    "peak_src": f"FP64 = {pk['src']} bf16 x nominal FP64/BF16 ratio (1.25/2250)",
+                    "peak_src": FP64_SRC,
                     "ms_per_evaluation": mp}
     else:
         # algorithmic bytes: the energy kernel reads each product output element once
@@ -663,11 +664,11 @@ def main():
     site, kms, kmacs = ctx.profile_top(reps=3)
     pk = peaks()
     if args.precision == "fp64":
-        peak = pk["bf16"] * FP64_NOMINAL_TFLOPS / BF16_NOMINAL_TFLOPS
+        peak = FP64_TFLOPS
         achieved = kmacs * 4 * 2 / (kms * 1e-3) / 1e12  # real FP64 flops: 4 real FMA per complex MAC
         roof = {"bound": "tensor", "kernel": f"k_gemm_fp64 ({site})", "achieved": achieved, "peak": peak,
                 "unit": "TFLOP/s", "frac": achieved / peak, "traffic": None,
-                "peak_src": f"FP64 = {pk['src']} bf16 x nominal FP64/BF16 ratio (1.25/2250)"}
+                "peak_src": FP64_SRC}
     else:
         pairs = smaj * (smaj + 1) // 2
         # executed BF16 tensor flops: 4 real MACs per complex MAC (real embedding; 1 in real
