@@ -56,11 +56,11 @@ __device__ __forceinline__ cplx pairwise(const cplx*& a, const cplx*& b, int64_t
 // (Loads of 8 terms ahead serve the few CTAs of 256 threads, 16 x 16 x 500000 1.30 -> 1.01
 // ms; where CTAs fill the chip 4 are better, 400 x 400 x 5000 5.74 -> 5.53 ms.)
 //
-// Measured against 64 x 64 shared-memory tiles
-// (with a warp per output for small products), TFLOP/s of complex work, exp_zgemm:
-// 1024^3 1.17 -> 1.22, 300^3 0.16 -> 0.81, 6000 x 24 x 400 0.27 -> 0.98, 64 x 64 x 5000
-// 0.14 -> 0.70; one CCSD iteration at o=10 v=40 8.2 -> 2.1 ms, at o=40 v=200 Z8 278 ->
-// 203 ms (1.22 TFLOP/s), (T) at o=24 v=120 Z8 1940 -> 97 ms.
+// Measured against 64 x 64 shared-memory tiles (with a warp per output for small
+// products), TFLOP/s of complex work, exp_zgemm calls: 1024^3 1.17 -> 1.22, 300^3 0.16 ->
+// 0.81, 6000 x 24 x 400 0.27 -> 0.98, 64 x 64 x 5000 0.14 -> 0.70 (the kernel alone: 1.23,
+// 1.09, 1.18, 1.10 of the pipe's 1.26); one CCSD iteration at o=10 v=40 8.2 -> 2.2 ms, at
+// o=40 v=200 Z8 278 -> 204 ms (1.21 TFLOP/s), (T) at o=24 v=120 Z8 1940 -> 95 ms.
 template <int THREADS, int LEAF>
 __global__ void __launch_bounds__(THREADS) k_gemm_fp64(const GemmProb* __restrict__ probs, int n_probs,
                                                        const cplx* __restrict__ A, const cplx* __restrict__ B,
